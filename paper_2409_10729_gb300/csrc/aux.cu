@@ -306,12 +306,14 @@ __global__ void conversion_check_kernel(long long n, unsigned long long seed, un
 
 // Self-check of the FP64 form's integer-pipe products K v and quotients x/6
 // against the FP64 instructions, and of its integer-word compares (x > 0,
-// 0 <= x, x < y) against the FP64 compares: pseudo-random patterns over every
+// 0 <= x, x < y) against the FP64 compares, and of the integer-pipe quotients
+// against the FP64 division: pseudo-random patterns over every
 // exponent, with a share of zeros, subnormals, infinities, NaNs and exponents
 // at the ends of the range where the integer path hands over to the FP64 one;
 // the second compare operand is another such pattern, x itself or x with its
 // lowest bit or its sign flipped.
 __global__ void exact_ops_check_kernel(long long n, unsigned long long seed, unsigned* mismatches) {
+    using namespace exact;
     unsigned bad = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
@@ -344,6 +346,22 @@ __global__ void exact_ops_check_kernel(long long n, unsigned long long seed, uns
         else if ((w & 7u) == 0u) w &= 0x8000000000000000ULL;   // +-0 now and then
         const double y = __longlong_as_double((long long)w);
         bad += (gt0(x) != (x > 0.0)) + (ge0(x) != (0.0 <= x)) + (less(x, y) != (x < y)) + (less(y, x) != (y < x));
+        // quotients from significands: operands moved into the range of
+        // mid_range, some with a significand next to a power of two, and the
+        // WENO5 linear weights as numerators
+        const unsigned long long me = (unsigned long long)(723 + (z >> 11) % 600) << 52;
+        unsigned long long fd = w & 0x000fffffffffffffULL, fn = (w * 0x9e3779b97f4a7c15ULL) >> 12;
+        const unsigned cut = (unsigned)(z >> 5) % 52u;
+        if (sel == 5) fd >>= cut;
+        else if (sel == 6) fd = ~(fd >> cut) & 0x000fffffffffffffULL;
+        else if (sel == 7) fn = fd;
+        else if (sel == 8) fn = (fd + (1ULL << cut)) & 0x000fffffffffffffULL;
+        const double den = __longlong_as_double((long long)(me | fd));
+        const double num = sel == 9    ? 0.1
+                           : sel == 10 ? 0.3
+                           : sel == 11 ? 0.6
+                                       : __longlong_as_double((long long)(((w >> 52) % 600 + 723) << 52 | fn));
+        bad += mid_range(den) && __double_as_longlong(quot_i(num, rcp_i(den))) != __double_as_longlong(num / den);
     }
     if (bad) atomicAdd(mismatches, bad);
 }
