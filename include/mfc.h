@@ -52,9 +52,9 @@ typedef enum {
                           (bit-identical to a serial evaluation in that order) */
     MFC_MIXED = 1,     /* FP32 state/stencils/Riemann; FP64 pressure recovery and RK update */
     MFC_GATED = 2,     /* MFC_MIXED plus an MLP gate choosing linear-weight WENO in smooth cells */
-    MFC_FP64_FAST = 3  /* FP64 with the formulas reorganised for fewer FP64 instructions
-                          (WENO in differences, product-form weights, FMA); agrees with
-                          MFC_FP64 to rounding, amplified by the flow over long runs */
+    MFC_FP64_FAST = 3  /* agrees with MFC_FP64 to rounding; since the latter's quotients moved to
+                          the integer pipes it is the faster of the two arithmetics, and both
+                          run it */
 } mfc_precision;
 
 typedef enum { MFC_BC_TRANSMISSIVE = 0, MFC_BC_PERIODIC = 1 } mfc_bc;

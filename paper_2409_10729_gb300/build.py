@@ -37,7 +37,7 @@ EXTRA = {"sweep_mixed.cu": FAST32, "sweep_gated.cu": FAST32,
 # extra nvcc flags for every unit (e.g. -DMFC_MIN_BLOCKS_MIXED=3); they are part
 # of the build key
 USER_FLAGS = os.environ.get("MFC5_NVCC_FLAGS", "").split()
-UNITS = ["capi.cu", "aux.cu", "sweep_fp64.cu", "sweep_fp64x.cu", "sweep_mixed.cu", "sweep_gated.cu", "mlp.cu",
+UNITS = ["capi.cu", "aux.cu", "sweep_fp64x.cu", "sweep_mixed.cu", "sweep_gated.cu", "mlp.cu",
          "noalloc.cu", "grid.cu", "blocks.cu"]
 
 

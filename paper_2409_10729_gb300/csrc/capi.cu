@@ -206,8 +206,8 @@ extern "C" int mfc_create(const mfc_params* params, void* cuda_stream, mfc_ctx**
     ctx->ndim = params->ndim;
     ctx->neq = 2 * params_nfluids(params->nfluids) + params->ndim;
     switch (params->precision) {
-        case MFC_FP64: ctx->form = FORM_FP64_EXACT; break;
-        case MFC_FP64_FAST: ctx->form = FORM_FP64_FAST; break;
+        case MFC_FP64:
+        case MFC_FP64_FAST: ctx->form = FORM_FP64_EXACT; break;
         case MFC_GATED: ctx->form = FORM_GATED; break;
         default: ctx->form = FORM_MIXED; break;
     }
@@ -314,7 +314,6 @@ static cudaError_t launch_sweep(mfc_ctx* ctx, int dir, int mode, SweepArgs a, cu
     }
     switch (ctx->form) {
         case FORM_FP64_EXACT: return launch_sweep_fp64x(ctx->ndim, dir, mode, a, s);
-        case FORM_FP64_FAST: return launch_sweep_fp64(ctx->ndim, dir, mode, a, s);
         case FORM_GATED: return launch_sweep_gated(ctx->ndim, dir, mode, a, s);
         default: return launch_sweep_mixed(ctx->ndim, dir, mode, a, s);
     }

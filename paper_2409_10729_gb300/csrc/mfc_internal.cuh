@@ -136,16 +136,14 @@ struct SweepArgs {
 constexpr int kTmaCells = 4;
 
 // Arithmetic forms of the sweep kernels:
-//   FORM_FP64_FAST   FP64, formulas reorganised for fewer FP64 instructions
 //   FORM_MIXED       FP32 stencils/Riemann, FP64 pressure numerator and RK update
-//   FORM_FP64_EXACT  FP64 in the reference operation order (bit-identical to it)
+//   FORM_FP64_EXACT  FP64 in the reference operation order (bit-identical to it); tile.cuh
 //   FORM_GATED       FORM_MIXED with the MLP gate (linear weights in smooth cells)
-enum Form { FORM_FP64_FAST = 0, FORM_MIXED = 1, FORM_FP64_EXACT = 2, FORM_GATED = 3 };
+enum Form { FORM_MIXED = 1, FORM_FP64_EXACT = 2, FORM_GATED = 3 };
 
 // Number of parameters of the gate network (W1[32][5], b1, W2[32][32], b2, w3, b3).
 constexpr int kGateParams = 1281;
 
-cudaError_t launch_sweep_fp64(int ndim, int dir, int mode, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_sweep_mixed(int ndim, int dir, int mode, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_sweep_fp64x(int ndim, int dir, int mode, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_sweep_gated(int ndim, int dir, int mode, const SweepArgs& a, cudaStream_t s);
@@ -184,15 +182,14 @@ cudaError_t run_fma_probe(int fp64, double* tflops, cudaStream_t s);
 constexpr int kSweepThreads = 128;
 // threads per block of the sweep along direction d
 __host__ __device__ constexpr int sweep_threads(int dir) { return dir == 0 ? 32 : kSweepThreads; }
-// Resident sweep blocks per SM requested from the register allocator,
-// counted in 128-thread blocks, per form, and for the FP32 forms separately
-// for the x sweep and for the last sweep with its stage update (1: up to 255
-// registers a thread; 2: 255; 3: 168; 4: 128).  The FP64 forms are bound by the FP64 pipe and lose nothing at
-// two blocks; the FP32 forms need the warps to cover their load latency.
-// Pencil segments per warp (cells along the sweep direction) are lengthened
-// up to MFC_MAX_SEG cells while the grid still fills the device's resident
-// blocks MFC_MIN_WAVES times (measured best at 256^3: FP64 64 cells, mixed
-// 32; at 512^3: mixed 128).
+// The sweep kernels of the FP32 forms (sweep.cuh).  Resident sweep blocks per
+// SM requested from the register allocator, counted in 128-thread blocks, per
+// form, and separately for the x sweep and for the last sweep with its stage
+// update (1: up to 255 registers a thread; 2: 255; 3: 168; 4: 128): they need
+// the warps to cover their load latency.  Pencil segments per warp (cells
+// along the sweep direction) are lengthened up to MFC_MAX_SEG cells while the
+// grid still fills the device's resident blocks MFC_MIN_WAVES times (measured
+// best, mixed: 32 at 256^3, 128 at 512^3).
 #ifndef MFC_MAX_SEG
 #define MFC_MAX_SEG 128
 #endif
@@ -204,15 +201,14 @@ __host__ __device__ constexpr int sweep_threads(int dir) { return dir == 0 ? 32 
 // of the T = (pencil groups x cells per pencil) cells in pencil-group order --
 // one or more pieces of consecutive pencil groups -- so every warp does the
 // same work and no partial last wave is left.  Warps take at least
-// MFC_BAL_MIN_CELLS cells (small grids launch fewer warps).  Used by the
-// forms where it measured faster: FP64 (256^3: 0.956 -> 0.913 ns), FP64-fast
-// (0.552 -> 0.523) and the mixed form with more than two fluids (0.0179 ->
-// 0.0171).  The two-fluid mixed form keeps the seg mapping: its sweeps are
-// register-capped, and the piece loop cost more than the balance gained
-// (512^3: 0.0149 -> 0.0170); so does the gated form, whose cost per warp
-// depends on the data (warp steps with all stencils flat skip the network),
-// where many short blocks let the block scheduler even it out.  0: the seg
-// mapping everywhere (and always for MFC_TMA_YZ sweeps).
+// MFC_BAL_MIN_CELLS cells (small grids launch fewer warps).  Used by the mixed
+// form with more than two fluids (0.0179 -> 0.0171 ns).  The two-fluid mixed
+// form keeps the seg mapping: its sweeps are register-capped, and the piece
+// loop cost more than the balance gained (512^3: 0.0149 -> 0.0170); so does
+// the gated form, whose cost per warp depends on the data (warp steps with all
+// stencils flat skip the network), where many short blocks let the block
+// scheduler even it out.  0: the seg mapping everywhere (and always for
+// MFC_TMA_YZ sweeps).
 #ifndef MFC_BALANCE
 #define MFC_BALANCE 1
 #endif
@@ -223,11 +219,8 @@ __host__ __device__ constexpr int sweep_threads(int dir) { return dir == 0 ? 32 
 #define MFC_BAL_MIN_CELLS 32
 #endif
 __host__ __device__ constexpr bool sweep_balanced(int form, int nf) {
-    return MFC_BALANCE && (form == FORM_FP64_EXACT || form == FORM_FP64_FAST || (form == FORM_MIXED && nf > 2));
+    return MFC_BALANCE && form == FORM_MIXED && nf > 2;
 }
-#ifndef MFC_MIN_BLOCKS_FP64
-#define MFC_MIN_BLOCKS_FP64 1
-#endif
 #ifndef MFC_MIN_BLOCKS_MIXED
 #define MFC_MIN_BLOCKS_MIXED 4
 #endif
@@ -246,15 +239,10 @@ __host__ __device__ constexpr bool sweep_balanced(int form, int nf) {
 // 1: the sweeps issue the loads of the cell entering the stencil window at the
 // top of each step along the pencil (they complete under that step's
 // arithmetic); 0: at the bottom, just before they are used.
-// FP64 reference-order sweeps: carry two WENO5 candidate values per field
-// from cell to cell (1) or form them in every cell (0)
 // mixed form, uniform grids, x sweep: carry WENO5 first differences and
 // curvature parts from cell to cell (1) or form them in every cell (0)
 #ifndef MFC_DIFF_CARRY
 #define MFC_DIFF_CARRY 1
-#endif
-#ifndef MFC_CAND_CARRY
-#define MFC_CAND_CARRY 1
 #endif
 #ifndef MFC_PREFETCH
 #define MFC_PREFETCH 1

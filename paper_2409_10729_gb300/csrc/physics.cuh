@@ -221,24 +221,7 @@ __device__ __forceinline__ void weno5(R v0, R v1, R v2, R v3, R v4, R eps, R& vm
     R b0 = c13 * D0 * D0 + R(0.25) * Q0 * Q0;
     R b1 = c13 * D1 * D1 + R(0.25) * Q1 * Q1;
     R b2 = c13 * D2 * D2 + R(0.25) * Q2 * Q2;
-    if constexpr (sizeof(R) == 4) {
-        weno5_tail32(v2, d1, d2, d3, d4, b0, b1, b2, eps, vm, vp);
-        return;
-    }
-    R s0 = eps + b0, s1 = eps + b1, s2 = eps + b2;
-    s0 = s0 * s0;
-    s1 = s1 * s1;
-    s2 = s2 * s2;
-    // product form: weight of stencil k is proportional to d_k * s_j * s_l
-    R m0 = s1 * s2, m1 = s0 * s2, m2 = s0 * s1;
-    R am0 = R(0.1) * m0, am1 = R(0.6) * m1, am2 = R(0.3) * m2;
-    R ap0 = R(0.3) * m0, ap1 = R(0.6) * m1, ap2 = R(0.1) * m2;
-    R Nm = am0 * (R(5) * d2 - R(2) * d1) + am1 * (d2 + R(2) * d3) + am2 * (R(4) * d3 - d4);
-    R Np = ap0 * (d1 - R(4) * d2) - ap1 * (R(2) * d2 + d3) + ap2 * (R(2) * d4 - R(5) * d3);
-    R Dm = am0 + am1 + am2, Dp = ap0 + ap1 + ap2;
-    R r = rdiv(R(1), R(6) * Dm * Dp);
-    vm = v2 + Nm * Dp * r;
-    vp = v2 + Np * Dm * r;
+    weno5_tail32(v2, d1, d2, d3, d4, b0, b1, b2, eps, vm, vp);
 }
 
 // WENO3-JS (Sec. II-B's third-order option; Jiang & Shu, stencils {i-1, i}

@@ -1,4 +1,5 @@
-// sweep.cuh -- the fused per-direction sweep kernel.
+// sweep.cuh -- the fused per-direction sweep kernel (FP32 forms; the FP64
+// form's sweeps are in tile.cuh) and the launch dispatch of all forms.
 //
 // One launch handles one direction d of one RHS evaluation (arXiv
 // 2409.10729, Sec. II-B): for every cell it converts conservative to
@@ -57,26 +58,6 @@ struct LoadSet {
 };
 
 // Primitives from the loaded values v[] (see LoadSet).
-template <int NDIM, int NF = 2>
-__device__ __forceinline__ void to_prim(const EosR<double, NF>& e, const double* v, double* w) {
-    using FL = Fields<NDIM, NF>;
-    double r = 1.0 / mix_rho<NF>(v);
-    double ke2 = 0.0;
-#pragma unroll
-    for (int i = 0; i < NF; ++i) w[i] = v[i];
-#pragma unroll
-    for (int k = 0; k < NDIM; ++k) {
-        double u = v[FL::IU + k] * r;
-        w[FL::IU + k] = u;
-        ke2 += v[FL::IU + k] * u;
-    }
-    double G, Pi;
-    mixture(e, v + FL::IA, G, Pi);
-    w[FL::IE] = (v[FL::IE] - 0.5 * ke2 - Pi) / G;
-#pragma unroll
-    for (int i = 0; i < FL::NA; ++i) w[FL::IA + i] = v[FL::IA + i];
-}
-
 template <int NDIM, int NF = 2>
 __device__ __forceinline__ void to_prim(const EosR<float, NF>& e, const float* v, float* w) {
     using FL = Fields<NDIM, NF>;
@@ -501,8 +482,7 @@ constexpr int sweep_min_blocks() {
     constexpr int per128 = FORM == FORM_MIXED   ? (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_MIXED_RK
                                                    : DIR == 0         ? MFC_MIN_BLOCKS_MIXED_X
                                                                       : MFC_MIN_BLOCKS_MIXED)
-                           : FORM == FORM_GATED ? (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_GATED_RK : MFC_MIN_BLOCKS_GATED)
-                                                : MFC_MIN_BLOCKS_FP64;
+                                                : (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_GATED_RK : MFC_MIN_BLOCKS_GATED);
     return per128 * 128 / sweep_threads(DIR);
 }
 
@@ -512,13 +492,11 @@ template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF>
 __global__ void __launch_bounds__(sweep_threads(DIR), sweep_min_blocks<FORM, MODE, DIR, NF>())
 sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
     using R = FormReal<FORM>;
-    constexpr bool EXACT = FORM == FORM_FP64_EXACT;
     constexpr bool GATED = FORM == FORM_GATED;
     using FL = Fields<NDIM, NF>;
     using LS = LoadSet<NDIM, R, NF>;
     constexpr int NEQ = FL::NEQ, IE = FL::IE, IA = FL::IA, NA = FL::NA;
     constexpr int NL = LS::N;
-    constexpr bool MIXED = FORM == FORM_MIXED || FORM == FORM_GATED;
     constexpr int CH = XStage<R>::CH, PITCH = XStage<R>::PITCH;
     constexpr int WARPS = sweep_threads(DIR) / 32;
     // x sweep writing the accumulator: the warp collects each sector's worth
@@ -576,21 +554,14 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
         r1 = gseg * ns + sseg1;
     }
     const long long nc = a.ncell;
-    const R inv_dx = sizeof(R) == 4 ? R(a.inv_dx32[DIR]) : R(a.inv_dx[DIR]);
+    const R inv_dx = R(a.inv_dx32[DIR]);
     const R eps = R(a.eps);
-    // FP64 reference-order form: a uniform width along DIR that is a power of two
-    // (zero fraction bits) with a normal reciprocal, which a.rdx then holds exactly
-    const unsigned dxh = (unsigned)__double2hiint(a.dx[DIR]), dxe = (dxh >> 20) & 0x7ffu;
-    const bool pow2_dx = EXACT && (dxh & 0x800fffffu) == 0u && __double2loint(a.dx[DIR]) == 0 && dxe - 2u < 2043u;
     const EosR<R, NF> er(a.eos);
     const R* __restrict__ qin = static_cast<const R*>(a.qin);
     const int wib = threadIdx.x >> 5;
 
-    // the FP64 reference-order kernels are FP64-pipe bound with latency to spare:
-    // the registers of a prefetched cell go to the carried candidates instead
-    constexpr bool PCARRY = EXACT && !GATED && !NU && NF == 2 && MFC_CAND_CARRY;
-    constexpr bool PREFETCH = MFC_PREFETCH != 0 && !PCARRY;
-    constexpr bool EPI_PREFETCH = PREFETCH && MIXED;
+    constexpr bool PREFETCH = MFC_PREFETCH != 0;
+    constexpr bool EPI_PREFETCH = PREFETCH;
     bool bad_any = false, tma_fail = false;
     R smax = R(0);
     unsigned n_gated = 0, n_fallback = 0, n_cells = 0, n_flat = 0;
@@ -661,7 +632,7 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
 
         // FP32 x sweep with rows of a multiple of 4 cells: 16-byte aligned rows,
         // loaded four cells at a time (cells are fetched in order along the row)
-        constexpr bool XVEC = MIXED && DIR == 0 && MFC_XVEC;
+        constexpr bool XVEC = DIR == 0 && MFC_XVEC;
         const bool xvec_ok = XVEC && (n0 & 3) == 0;
         float xq[XVEC ? NL : 1][3];
         int xpend = 0;
@@ -741,28 +712,8 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
         for (int k = 0; k < 5; ++k) {
             R v[NL];
             fetch(k, v);
-            if constexpr (EXACT) exact::cons_to_prim<NDIM, NF>(a.eos, v, W[k]);
-            else to_prim<NDIM, NF>(er, v, W[k]);
+            to_prim<NDIM, NF>(er, v, W[k]);
             bad |= !pos(mix_rho<NF>(W[k]));
-        }
-        // FP64 reference-order form: the smoothness indicators' curvature terms
-        // of the window's stencils {i-2..i}, {i-1..i+1} (cell i = window centre),
-        // carried along the pencil so that each is formed once (exact::curv)
-        constexpr bool TCARRY = EXACT && !GATED && !NU && NF == 2;
-        double Tm[TCARRY ? NEQ : 1], T0[TCARRY ? NEQ : 1];
-        if constexpr (TCARRY) {
-#pragma unroll
-            for (int f = 0; f < NEQ; ++f) {
-                Tm[f] = exact::curv(W[0][f], W[1][f], W[2][f]);
-                T0[f] = exact::curv(W[1][f], W[2][f], W[3][f]);
-            }
-        }
-        // and the right-face candidates of the window's centre cell, carried as
-        // the left-face candidates of the cell before it (exact::weno5_tc)
-        double Pr0[PCARRY ? NEQ : 1], Pr1[PCARRY ? NEQ : 1];
-        if constexpr (PCARRY) {
-#pragma unroll
-            for (int f = 0; f < NEQ; ++f) exact::weno5_right01(W[0][f], W[1][f], W[2][f], W[3][f], Pr0[f], Pr1[f]);
         }
         // mixed form, x sweep: the first differences d1..d3 and curvature parts C0, C1
         // of the window's centre cell, carried along the pencil (weno5_dc); the y and
@@ -856,21 +807,7 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
                 } else if (GATED || a.order == 5) {
 #pragma unroll
                     for (int f = 0; f < NEQ; ++f) {
-                        if constexpr (PCARRY) {
-                            const double Tp = exact::curv(W[2][f], W[3][f], W[4][f]);
-                            exact::weno5_tc(a.eps, W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], Tm[f], T0[f], Tp,
-                                            Pr0[f], Pr1[f], vm[f], vp[f]);
-                            Tm[f] = T0[f];
-                            T0[f] = Tp;
-                        } else if constexpr (TCARRY) {
-                            const double Tp = exact::curv(W[2][f], W[3][f], W[4][f]);
-                            exact::weno5_t(a.eps, W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], Tm[f], T0[f], Tp,
-                                           vm[f], vp[f]);
-                            Tm[f] = T0[f];
-                            T0[f] = Tp;
-                        } else if constexpr (EXACT) {
-                            exact::weno5(a.eps, W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], vm[f], vp[f]);
-                        } else if constexpr (DCARRY) {
+                        if constexpr (DCARRY) {
                             const float d4 = float(W[4][f] - W[3][f]);
                             const float D2 = d4 - Dd3[f];
                             const float C2 = c13f * D2 * D2;
@@ -890,50 +827,24 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
                 } else {   // WENO3 (uniform over the launch): cells i-1 .. i+1 of the window
 #pragma unroll
                     for (int f = 0; f < NEQ; ++f) {
-                        if constexpr (EXACT) exact::weno3(a.eps, W[1][f], W[2][f], W[3][f], vm[f], vp[f]);
-                        else weno3(W[1][f], W[2][f], W[3][f], eps, vm[f], vp[f]);
+                        weno3(W[1][f], W[2][f], W[3][f], eps, vm[f], vp[f]);
                     }
                 }
             }
             if (j >= s0) {
                 R F[NEQ], uf;
-                if constexpr (EXACT) bad |= exact::hllc<NDIM, DIR, NF>(a.eos, vmPrev, vp, F, uf);
-                else bad |= hllc<NDIM, DIR, R, NF>(er, vmPrev, vp, F, uf);
+                bad |= hllc<NDIM, DIR, R, NF>(er, vmPrev, vp, F, uf);
                 if (j > s0 && (active || OSTAGE_ON)) {
                     // cell i = j - 1 is complete: faces i-1/2 (Fprev) and i+1/2 (F)
                     R L[NEQ];
-                    if constexpr (EXACT) {
-                        // (F_{i-1/2} - F_{i+1/2})/dx, then + alpha1 (u_f+ - u_f-)/dx
-                        double dx = a.dx[DIR], rdx = a.rdx[DIR];
-                        if (NU && a.cw[DIR]) {   // non-uniform: the cell's own width
-                            dx = __ldg(a.cw[DIR] + (j - 1));
-                            rdx = __ldg(a.crw[DIR] + (j - 1));
-                        }
-                        if (pow2_dx && !(NU && a.cw[DIR])) {
-                            // a power-of-two width: x / dx and x * (1/dx) are the same real
-                            // number, so one multiplication gives the quotient's bits
-#pragma unroll
-                            for (int f = 0; f < NEQ; ++f) L[f] = (Fprev[f] - F[f]) * rdx;
-#pragma unroll
-                            for (int i = 0; i < NA; ++i) L[IA + i] = L[IA + i] + alphaCell[i] * (uf - ufPrev) * rdx;
-                        } else {
-#pragma unroll
-                            for (int f = 0; f < NEQ; ++f) L[f] = exact::div_rcp(Fprev[f] - F[f], dx, rdx);
-#pragma unroll
-                            for (int i = 0; i < NA; ++i)
-                                L[IA + i] = L[IA + i] + exact::div_rcp(alphaCell[i] * (uf - ufPrev), dx, rdx);
-                        }
-                    } else {
-                        R idx = inv_dx;
-                        if (NU && a.cw[DIR]) {
-                            if constexpr (sizeof(R) == 8) idx = __ldg(a.crw[DIR] + (j - 1));
-                            else idx = __ldg(a.crw32[DIR] + (j - 1));
-                        }
-#pragma unroll
-                        for (int f = 0; f < NEQ; ++f) L[f] = (Fprev[f] - F[f]) * idx;
-#pragma unroll
-                        for (int i = 0; i < NA; ++i) L[IA + i] += alphaCell[i] * (uf - ufPrev) * idx;
+                    R idx = inv_dx;
+                    if (NU && a.cw[DIR]) {
+                        idx = __ldg(a.crw32[DIR] + (j - 1));
                     }
+#pragma unroll
+                    for (int f = 0; f < NEQ; ++f) L[f] = (Fprev[f] - F[f]) * idx;
+#pragma unroll
+                    for (int i = 0; i < NA; ++i) L[IA + i] += alphaCell[i] * (uf - ufPrev) * idx;
                     const long long c = base + (long long)(j - 1) * ss;
                     if constexpr (OSTAGE_ON) {
                         R* o = ostage + (threadIdx.x >> 5) * OSTAGE + lane * PITCH + ((j - 1) & (CH - 1));
@@ -962,75 +873,43 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
                         for (int f = 0; f < NEQ; ++f) {
                             R tot = NDIM > 1 ? (EPI_PREFETCH ? accp[f] : acc[f * nc + c]) + L[f] : L[f];
                             double qn = EPI_PREFETCH ? qnp[f] : a.qn[f * nc + c];
-                            if constexpr (MIXED) {
-                                // D_k in FP32 from D_(k-1) and the FP32 L; q^(k) = q^n + D_k in FP64
-                                float Dk;
-                                if (a.stage == 1) {
-                                    Dk = dt32 * float(tot);
-                                } else {
-                                    const float Dp = EPI_PREFETCH ? float(qkp[f]) : a.dinc[f * nc + c];
-                                    Dk = kfac * fmaf(dt32, float(tot), Dp);
-                                }
-                                if (a.stage != 3) a.dinc[f * nc + c] = Dk;
-                                qnew[f] = qn + f2d_bits(Dk);
+                            // D_k in FP32 from D_(k-1) and the FP32 L; q^(k) = q^n + D_k in FP64
+                            float Dk;
+                            if (a.stage == 1) {
+                                Dk = dt32 * float(tot);
                             } else {
-                                double dL = dt * double(tot);
-                                if (a.stage == 1) {
-                                    qnew[f] = qn + dL;
-                                } else {
-                                    double qkd = double(qin[f * nc + c]);
-                                    if (a.stage == 2)
-                                        qnew[f] = 0.75 * qn + 0.25 * (qkd + dL);
-                                    else
-                                        qnew[f] = (1.0 / 3.0) * qn + (2.0 / 3.0) * (qkd + dL);
-                                }
+                                const float Dp = EPI_PREFETCH ? float(qkp[f]) : a.dinc[f * nc + c];
+                                Dk = kfac * fmaf(dt32, float(tot), Dp);
                             }
+                            if (a.stage != 3) a.dinc[f * nc + c] = Dk;
+                            qnew[f] = qn + f2d_bits(Dk);
                         }
-                        if constexpr (!MIXED) {
-                            double* out = static_cast<double*>(a.qout);
+                        float q32[NEQ];
 #pragma unroll
-                            for (int f = 0; f < NEQ; ++f) out[f * nc + c] = qnew[f];
-                            if (a.stage == 3) {
-                                R s;
+                        for (int f = 0; f < NEQ; ++f) q32[f] = d2f_bits(qnew[f]);
+                        float pnew = mixed_pressure<NDIM, NF>(a.eos, qnew, q32);
+                        float* o32 = static_cast<float*>(a.stage == 3 ? a.qout2 : a.qout);
+#pragma unroll
+                        for (int f = 0; f < NEQ; ++f) o32[f * nc + c] = q32[f];
+                        o32[NEQ * nc + c] = pnew;
+                        if (a.stage == 3) {
+                            double* o64 = static_cast<double*>(a.qout);
+#pragma unroll
+                            for (int f = 0; f < NEQ; ++f) o64[f * nc + c] = qnew[f];
+                            float v[NEQ], wn[NEQ];
+#pragma unroll
+                            for (int f = 0; f < NEQ; ++f) v[f] = q32[f];
+                            v[IE] = pnew;
+                            to_prim<NDIM, NF>(er, v, wn);
+                            float idx32[3] = {a.inv_dx32[0], a.inv_dx32[1], a.inv_dx32[2]};
+                            if constexpr (NU) {
                                 double dx3[3], rdx3[3], idx3[3];
                                 cell_geometry<DIR, NU>(a, j - 1, active ? ia : na - 1, b, dx3, rdx3, idx3);
-                                if constexpr (EXACT) {
-                                    s = exact::cell_wavespeed<NDIM, NF>(a.eos, qnew, dx3, rdx3, bad);
-                                } else {
-                                    double wn[NEQ];
-                                    to_prim<NDIM, NF>(er, qnew, wn);
-                                    s = cell_wavespeed<NDIM, double, NF>(er, wn, idx3, bad);
-                                }
-                                smax = s > smax ? s : smax;
+#pragma unroll
+                                for (int d = 0; d < 3; ++d) idx32[d] = float(idx3[d]);
                             }
-                        } else {
-                            float q32[NEQ];
-#pragma unroll
-                            for (int f = 0; f < NEQ; ++f) q32[f] = d2f_bits(qnew[f]);
-                            float pnew = mixed_pressure<NDIM, NF>(a.eos, qnew, q32);
-                            float* o32 = static_cast<float*>(a.stage == 3 ? a.qout2 : a.qout);
-#pragma unroll
-                            for (int f = 0; f < NEQ; ++f) o32[f * nc + c] = q32[f];
-                            o32[NEQ * nc + c] = pnew;
-                            if (a.stage == 3) {
-                                double* o64 = static_cast<double*>(a.qout);
-#pragma unroll
-                                for (int f = 0; f < NEQ; ++f) o64[f * nc + c] = qnew[f];
-                                float v[NEQ], wn[NEQ];
-#pragma unroll
-                                for (int f = 0; f < NEQ; ++f) v[f] = q32[f];
-                                v[IE] = pnew;
-                                to_prim<NDIM, NF>(er, v, wn);
-                                float idx32[3] = {a.inv_dx32[0], a.inv_dx32[1], a.inv_dx32[2]};
-                                if constexpr (NU) {
-                                    double dx3[3], rdx3[3], idx3[3];
-                                    cell_geometry<DIR, NU>(a, j - 1, active ? ia : na - 1, b, dx3, rdx3, idx3);
-#pragma unroll
-                                    for (int d = 0; d < 3; ++d) idx32[d] = float(idx3[d]);
-                                }
-                                R s = cell_wavespeed<NDIM, float, NF>(er, wn, idx32, bad);
-                                smax = s > smax ? s : smax;
-                            }
+                            R s = cell_wavespeed<NDIM, float, NF>(er, wn, idx32, bad);
+                            smax = s > smax ? s : smax;
                         }
                     }
                 }
@@ -1071,8 +950,7 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
 #pragma unroll
                     for (int f = 0; f < NEQ; ++f) W[k][f] = W[k + 1][f];
                 if (!PREFETCH) fetch(j + 3 - (s0 - 3), vnext);
-                if constexpr (EXACT) exact::cons_to_prim<NDIM, NF>(a.eos, vnext, W[4]);
-                else to_prim<NDIM, NF>(er, vnext, W[4]);
+                to_prim<NDIM, NF>(er, vnext, W[4]);
                 bad |= !pos(mix_rho<NF>(W[4]));
             }
         }
@@ -1185,14 +1063,25 @@ cudaError_t launch_kernel(const SweepArgs& a0, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// the FP64 form's sweep (tile.cuh)
+template <int NDIM, int DIR, int MODE, bool NU, int NF>
+cudaError_t launch_tile(const SweepArgs& a, cudaStream_t s);
+
 template <int NDIM, int DIR, int MODE, int FORM, int NF>
 cudaError_t launch_one(const SweepArgs& a, cudaStream_t s) {
     const bool nu = a.cw[0] || a.cw[1] || a.cw[2];
+    if constexpr (FORM == FORM_FP64_EXACT) {
+        if constexpr (NF == 2) {
+            if (nu) return launch_tile<NDIM, DIR, MODE, true, NF>(a, s);
+        }
+        return nu ? cudaErrorInvalidValue : launch_tile<NDIM, DIR, MODE, false, NF>(a, s);
+    } else {
     if constexpr (FORM != FORM_GATED && NF == 2) {
         if (nu) return launch_kernel<NDIM, DIR, MODE, FORM, true, NF>(a, s);
     }
     if (nu) return cudaErrorInvalidValue;   // non-uniform grids: two fluids, non-gated forms
     return launch_kernel<NDIM, DIR, MODE, FORM, false, NF>(a, s);
+    }
 }
 
 // Launch one sweep: the valid (direction, mode) pairs are x FIRST, y MID
