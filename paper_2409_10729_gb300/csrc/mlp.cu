@@ -31,112 +31,164 @@ static_assert(kMlpParams == 1281, "parameter layout");
 
 __device__ __forceinline__ float softplusf(float t) { return t > 0.f ? t + log1pf(expf(-t)) : log1pf(expf(t)); }
 
-// Loss and gradient over n samples.  Block = kGradThreads threads; each pass
-// of a block takes kGradThreads samples: one thread per sample runs the
-// forward and backward pass and stages its activations in shared memory,
-// then every thread accumulates ~10 parameters over the staged samples.
-// Block partial sums go to global memory with one atomic add per parameter.
-constexpr int kGradThreads = 128;
-constexpr int kStage = kMlpIn + 4 * kMlpH + 1;  // x, h1, d1, d2, dz*h2, dz
+// Loss and gradient over n samples.  Lane l of a warp is neuron l: it holds row
+// l of W1 and W2, column l of W2 and the gradient sums of row l of W1, column l
+// of W2 and its biases in registers, and a warp takes four samples at a time
+// through both passes.  What every lane needs of the others (h1 for the forward
+// pass, d2 for the backward one) goes through 512 bytes of the warp's own
+// shared memory, read as broadcast 16-byte words: one such load feeds four
+// FMAs forward, and eight backward (d1 and dW2).  A block's warps add their sums in
+// shared memory, one atomic per parameter and block follows.  One block per
+// SM: a batch of 8192 gives a warp four or eight samples, and more blocks would
+// only add atomics (64 blocks: 14.5 us a call).  Measured per call with the
+// zeroing, batch 8192: 20.5 us with one thread per sample, its activations in
+// local memory and 128 samples per block, 10.4 now, of which the launches'
+// latencies are about half.
+constexpr int kGradWarps = 8, kGradGroup = 4;
 
-__global__ void __launch_bounds__(kGradThreads)
+__global__ void __launch_bounds__(kGradWarps * 32)
 mlp_grad_kernel(const float* __restrict__ X, const float* __restrict__ Y, long long n,
                 const float* __restrict__ theta, float wp, float inv_n, float* grad, float* loss) {
-    extern __shared__ float sm[];
-    float* th = sm;                        // kMlpParams
-    float* st = sm + kMlpParams;           // kGradThreads * kStage
-    for (int k = threadIdx.x; k < kMlpParams; k += blockDim.x) th[k] = theta[k];
+    __shared__ float part[kGradWarps][kMlpParams + 1];   // and the loss
+    __shared__ float4 act[kGradWarps][kGradGroup][kMlpH / 4];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    // the weights come through shared memory (W2 in rows of 33, so that rows and
+    // columns are read without bank conflicts): read from global memory by every
+    // lane, the rows alone cost 8192 L1 accesses per block
+    float* th = part[0];
+    for (int k = threadIdx.x; k < kMlpParams; k += blockDim.x) {
+        const int o = k < OW2 || k >= OB2 ? k : OW2 + (k - OW2) / kMlpH * (kMlpH + 1) + (k - OW2) % kMlpH;
+        th[o + (k >= OB2 ? kMlpH : 0)] = __ldg(theta + k);
+    }
     __syncthreads();
-    constexpr int PER = (kMlpParams + kGradThreads - 1) / kGradThreads;
-    float acc[PER];
+    float w1[kMlpIn], w2r[kMlpH], w2c[kMlpH];
 #pragma unroll
-    for (int r = 0; r < PER; ++r) acc[r] = 0.f;
-    float lsum = 0.f;
-    for (long long base = (long long)blockIdx.x * kGradThreads; base < n;
-         base += (long long)gridDim.x * kGradThreads) {
-        long long s = base + threadIdx.x;
-        float* me = st + threadIdx.x * kStage;
-        if (s < n) {
-            float x[kMlpIn], h1[kMlpH], h2[kMlpH], d2[kMlpH];
+    for (int i = 0; i < kMlpIn; ++i) w1[i] = th[OW1 + lane * kMlpIn + i];
 #pragma unroll
-            for (int i = 0; i < kMlpIn; ++i) x[i] = X[s * kMlpIn + i];
-#pragma unroll 4
-            for (int j = 0; j < kMlpH; ++j) {
-                float a = th[OB1 + j];
-#pragma unroll
-                for (int i = 0; i < kMlpIn; ++i) a = fmaf(th[OW1 + j * kMlpIn + i], x[i], a);
-                h1[j] = fmaxf(a, 0.f);
-            }
-#pragma unroll 4
-            for (int j = 0; j < kMlpH; ++j) {
-                float a = th[OB2 + j];
-#pragma unroll
-                for (int i = 0; i < kMlpH; ++i) a = fmaf(th[OW2 + j * kMlpH + i], h1[i], a);
-                h2[j] = fmaxf(a, 0.f);
-            }
-            float z = th[OB3];
-#pragma unroll
-            for (int i = 0; i < kMlpH; ++i) z = fmaf(th[OW3 + i], h2[i], z);
-            float y = Y[s];
-            lsum += wp * y * softplusf(-z) + (1.f - y) * softplusf(z);
-            float sg = 1.f / (1.f + expf(-z));
-            float dz = (wp * y * (sg - 1.f) + (1.f - y) * sg) * inv_n;
-#pragma unroll
-            for (int i = 0; i < kMlpH; ++i) d2[i] = h2[i] > 0.f ? dz * th[OW3 + i] : 0.f;
-#pragma unroll
-            for (int i = 0; i < kMlpIn; ++i) me[i] = x[i];
-#pragma unroll 4
-            for (int i = 0; i < kMlpH; ++i) {
-                float a = 0.f;
-#pragma unroll
-                for (int j = 0; j < kMlpH; ++j) a = fmaf(th[OW2 + j * kMlpH + i], d2[j], a);
-                me[kMlpIn + i] = h1[i];
-                me[kMlpIn + kMlpH + i] = h1[i] > 0.f ? a : 0.f;
-                me[kMlpIn + 2 * kMlpH + i] = d2[i];
-                me[kMlpIn + 3 * kMlpH + i] = dz * h2[i];
-            }
-            me[kStage - 1] = dz;
-        } else {
-            for (int i = 0; i < kStage; ++i) me[i] = 0.f;
-        }
-        __syncthreads();
-        // parameter k: sum over the staged samples of its per-sample gradient
-#pragma unroll
-        for (int r = 0; r < PER; ++r) {
-            int k = threadIdx.x + r * kGradThreads;
-            if (k >= kMlpParams) break;
-            float a = acc[r];
-            if (k < OB1) {                 // W1[j][i] += d1_j x_i
-                int j = k / kMlpIn, i = k % kMlpIn;
-                for (int t = 0; t < kGradThreads; ++t) a = fmaf(st[t * kStage + kMlpIn + kMlpH + j], st[t * kStage + i], a);
-            } else if (k < OW2) {          // b1[j] += d1_j
-                int j = k - OB1;
-                for (int t = 0; t < kGradThreads; ++t) a += st[t * kStage + kMlpIn + kMlpH + j];
-            } else if (k < OB2) {          // W2[j][i] += d2_j h1_i
-                int j = (k - OW2) / kMlpH, i = (k - OW2) % kMlpH;
-                for (int t = 0; t < kGradThreads; ++t)
-                    a = fmaf(st[t * kStage + kMlpIn + 2 * kMlpH + j], st[t * kStage + kMlpIn + i], a);
-            } else if (k < OW3) {          // b2[j] += d2_j
-                int j = k - OB2;
-                for (int t = 0; t < kGradThreads; ++t) a += st[t * kStage + kMlpIn + 2 * kMlpH + j];
-            } else if (k < OB3) {          // w3[i] += dz h2_i
-                int i = k - OW3;
-                for (int t = 0; t < kGradThreads; ++t) a += st[t * kStage + kMlpIn + 3 * kMlpH + i];
-            } else {                       // b3 += dz
-                for (int t = 0; t < kGradThreads; ++t) a += st[t * kStage + kStage - 1];
-            }
-            acc[r] = a;
-        }
-        __syncthreads();
+    for (int i = 0; i < kMlpH; ++i) {
+        w2r[i] = th[OW2 + lane * (kMlpH + 1) + i];
+        w2c[i] = th[OW2 + i * (kMlpH + 1) + lane];
     }
+    const float b1 = th[OB1 + lane], b2 = th[OB2 + kMlpH + lane], w3 = th[OW3 + kMlpH + lane];
+    const float b3 = th[OB3 + kMlpH];
+    __syncthreads();   // part is written again at the end
+    float g1[kMlpIn] = {}, g2[kMlpH] = {}, gb1 = 0.f, gb2 = 0.f, g3 = 0.f, gb3 = 0.f, lsum = 0.f;
+    float4(*my)[kMlpH / 4] = act[wib];
+    const long long step = (long long)gridDim.x * kGradWarps * kGradGroup;
+    for (long long base = ((long long)blockIdx.x * kGradWarps + wib) * kGradGroup; base < n; base += step) {
+        float x[kGradGroup][kMlpIn], h1[kGradGroup], h2[kGradGroup], z[kGradGroup], dz[kGradGroup];
 #pragma unroll
-    for (int r = 0; r < PER; ++r) {
-        int k = threadIdx.x + r * kGradThreads;
-        if (k < kMlpParams) atomicAdd(&grad[k], acc[r]);
+        for (int s = 0; s < kGradGroup; ++s) {
+            const long long k = base + s < n ? base + s : n - 1;   // past the end: weight 0 below
+            float a = b1;
+#pragma unroll
+            for (int i = 0; i < kMlpIn; ++i) {
+                x[s][i] = __ldg(X + k * kMlpIn + i);
+                a = fmaf(w1[i], x[s][i], a);
+            }
+            h1[s] = fmaxf(a, 0.f);
+            reinterpret_cast<float*>(my[s])[lane] = h1[s];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < kGradGroup; ++s) {
+            float a = b2;
+#pragma unroll
+            for (int q = 0; q < kMlpH / 4; ++q) {
+                const float4 v = my[s][q];
+                a = fmaf(w2r[4 * q], v.x, a);
+                a = fmaf(w2r[4 * q + 1], v.y, a);
+                a = fmaf(w2r[4 * q + 2], v.z, a);
+                a = fmaf(w2r[4 * q + 3], v.w, a);
+            }
+            h2[s] = fmaxf(a, 0.f);
+            z[s] = w3 * h2[s];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int s = 0; s < kGradGroup; ++s) z[s] += __shfl_xor_sync(0xffffffffu, z[s], o);
+        // lane s finishes sample s (every lane holds the sums)
+        {
+            const int s = lane & (kGradGroup - 1);
+            float zs = z[0];
+#pragma unroll
+            for (int k = 1; k < kGradGroup; ++k) zs = s == k ? z[k] : zs;
+            zs += b3;
+            const bool in = base + s < n;
+            const float y = __ldg(Y + (in ? base + s : n - 1));
+            const float sg = 1.f / (1.f + expf(-zs));
+            const float d = in ? (wp * y * (sg - 1.f) + (1.f - y) * sg) * inv_n : 0.f;
+            if (lane < kGradGroup) {
+                gb3 += d;
+                if (in) lsum += wp * y * softplusf(-zs) + (1.f - y) * softplusf(zs);
+            }
+#pragma unroll
+            for (int k = 0; k < kGradGroup; ++k) dz[k] = __shfl_sync(0xffffffffu, d, k);
+        }
+        __syncwarp();   // h1 has been read by every lane
+#pragma unroll
+        for (int s = 0; s < kGradGroup; ++s) {
+            const float d2 = h2[s] > 0.f ? dz[s] * w3 : 0.f;
+            reinterpret_cast<float*>(my[s])[lane] = d2;
+            gb2 += d2;
+            g3 = fmaf(dz[s], h2[s], g3);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int s = 0; s < kGradGroup; ++s) {
+            float a = 0.f;
+#pragma unroll
+            for (int q = 0; q < kMlpH / 4; ++q) {
+                const float4 v = my[s][q];
+                a = fmaf(w2c[4 * q], v.x, a);
+                a = fmaf(w2c[4 * q + 1], v.y, a);
+                a = fmaf(w2c[4 * q + 2], v.z, a);
+                a = fmaf(w2c[4 * q + 3], v.w, a);
+                g2[4 * q] = fmaf(v.x, h1[s], g2[4 * q]);
+                g2[4 * q + 1] = fmaf(v.y, h1[s], g2[4 * q + 1]);
+                g2[4 * q + 2] = fmaf(v.z, h1[s], g2[4 * q + 2]);
+                g2[4 * q + 3] = fmaf(v.w, h1[s], g2[4 * q + 3]);
+            }
+            const float d1 = h1[s] > 0.f ? a : 0.f;
+            gb1 += d1;
+#pragma unroll
+            for (int i = 0; i < kMlpIn; ++i) g1[i] = fmaf(d1, x[s][i], g1[i]);
+        }
+        __syncwarp();   // d2 has been read before the next samples' h1 is written
     }
-    // loss: warp reduction, then one atomic per warp
-    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, lsum * inv_n);
+    float* mine = part[wib];
+#pragma unroll
+    for (int i = 0; i < kMlpIn; ++i) mine[OW1 + lane * kMlpIn + i] = g1[i];
+#pragma unroll
+    for (int j = 0; j < kMlpH; ++j) mine[OW2 + j * kMlpH + lane] = g2[j];
+    mine[OB1 + lane] = gb1;
+    mine[OB2 + lane] = gb2;
+    mine[OW3 + lane] = g3;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        gb3 += __shfl_xor_sync(0xffffffffu, gb3, o);
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    }
+    if (lane == 0) {
+        mine[OB3] = gb3;
+        mine[kMlpParams] = lsum;
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k <= kMlpParams; k += blockDim.x) {
+        float a = part[0][k];
+#pragma unroll
+        for (int w = 1; w < kGradWarps; ++w) a += part[w][k];
+        if (k < kMlpParams) atomicAdd(&grad[k], a);
+        else atomicAdd(loss, a * inv_n);
+    }
+}
+
+// grad and loss start from zero
+__global__ void mlp_zero_kernel(float* grad, float* loss) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < kMlpParams) grad[k] = 0.f;
+    if (k == kMlpParams) *loss = 0.f;
 }
 
 __global__ void mlp_adam_kernel(float* theta, const float* __restrict__ g, float* m, float* v, float lr, float b1,
@@ -151,38 +203,52 @@ __global__ void mlp_adam_kernel(float* theta, const float* __restrict__ g, float
     theta[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
 }
 
-// Logit of one normalised stencil x[5] with parameters th (any memory space).
-__device__ __forceinline__ float mlp_logit(const float* th, const float* x) {
-    float h1[kMlpH];
-#pragma unroll 4
-    for (int j = 0; j < kMlpH; ++j) {
-        float a = th[OB1 + j];
-#pragma unroll
-        for (int i = 0; i < kMlpIn; ++i) a = fmaf(th[OW1 + j * kMlpIn + i], x[i], a);
-        h1[j] = fmaxf(a, 0.f);
+// Logits: one thread per sample, activations in registers (both layers fully
+// unrolled), weight rows read from shared memory as broadcast 16-byte words --
+// four FMAs a load, where one-word loads bound the kernel.
+__global__ void __launch_bounds__(128) mlp_forward_kernel(const float* __restrict__ X, long long n,
+                                                          const float* __restrict__ theta, float* z) {
+    __shared__ float4 w2[kMlpH][kMlpH / 4];
+    __shared__ float4 w1[kMlpH][2];   // W1[j][0..4], b1[j], b2[j], w3[j]
+    for (int k = threadIdx.x; k < kMlpH * kMlpH; k += blockDim.x)
+        reinterpret_cast<float*>(w2)[k] = __ldg(theta + OW2 + k);
+    for (int k = threadIdx.x; k < kMlpH * 8; k += blockDim.x) {
+        const int j = k >> 3, i = k & 7;
+        reinterpret_cast<float*>(w1)[k] =
+            __ldg(theta + (i < kMlpIn ? OW1 + j * kMlpIn + i : (i == 5 ? OB1 : (i == 6 ? OB2 : OW3)) + j));
     }
-    float z = th[OB3];
-#pragma unroll 2
-    for (int j = 0; j < kMlpH; ++j) {
-        float a = th[OB2 + j];
-#pragma unroll
-        for (int i = 0; i < kMlpH; ++i) a = fmaf(th[OW2 + j * kMlpH + i], h1[i], a);
-        z = fmaf(th[OW3 + j], fmaxf(a, 0.f), z);
-    }
-    return z;
-}
-
-__global__ void mlp_forward_kernel(const float* __restrict__ X, long long n, const float* __restrict__ theta,
-                                   float* z) {
-    __shared__ float th[kMlpParams];
-    for (int k = threadIdx.x; k < kMlpParams; k += blockDim.x) th[k] = theta[k];
     __syncthreads();
+    const float b3 = __ldg(theta + OB3);
     for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n;
          s += (long long)gridDim.x * blockDim.x) {
-        float x[kMlpIn];
+        float x[kMlpIn], h[kMlpH];
 #pragma unroll
-        for (int i = 0; i < kMlpIn; ++i) x[i] = X[s * kMlpIn + i];
-        z[s] = mlp_logit(th, x);
+        for (int i = 0; i < kMlpIn; ++i) x[i] = __ldg(X + s * kMlpIn + i);
+#pragma unroll
+        for (int j = 0; j < kMlpH; ++j) {
+            const float4 a = w1[j][0], b = w1[j][1];
+            float v = fmaf(a.x, x[0], b.y);
+            v = fmaf(a.y, x[1], v);
+            v = fmaf(a.z, x[2], v);
+            v = fmaf(a.w, x[3], v);
+            h[j] = fmaxf(fmaf(b.x, x[4], v), 0.f);
+        }
+        float out = b3;
+#pragma unroll 4
+        for (int j = 0; j < kMlpH; ++j) {
+            const float4 b = w1[j][1];
+            float v = b.z;
+#pragma unroll
+            for (int q = 0; q < kMlpH / 4; ++q) {
+                const float4 w = w2[j][q];
+                v = fmaf(w.x, h[4 * q], v);
+                v = fmaf(w.y, h[4 * q + 1], v);
+                v = fmaf(w.z, h[4 * q + 2], v);
+                v = fmaf(w.w, h[4 * q + 3], v);
+            }
+            out = fmaf(b.w, fmaxf(v, 0.f), out);
+        }
+        z[s] = out;
     }
 }
 
@@ -274,20 +340,12 @@ extern "C" int mfc_mlp_loss_grad(const float* X, const float* Y, long long n, co
                                  float* grad, float* loss, void* cuda_stream) {
     if (!X || !Y || !theta || !grad || !loss || n <= 0 || !(pos_weight > 0.f)) return MFC_EINVAL;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const size_t smem = sizeof(float) * (kMlpParams + kGradThreads * kStage);
-    static bool attr = false;
-    if (!attr) {
-        if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-            cudaSuccess)
-            return MFC_ECUDA;
-        attr = true;
-    }
-    if (cudaMemsetAsync(grad, 0, sizeof(float) * kMlpParams, s) != cudaSuccess ||
-        cudaMemsetAsync(loss, 0, sizeof(float), s) != cudaSuccess)
-        return MFC_ECUDA;
-    long long blocks = (n + kGradThreads - 1) / kGradThreads;
-    if (blocks > 152LL * 2) blocks = 152LL * 2;
-    mlp_grad_kernel<<<(unsigned)blocks, kGradThreads, smem, s>>>(X, Y, n, theta, pos_weight, 1.0f / (float)n, grad,
+    mlp_zero_kernel<<<(kMlpParams + 256) / 256, 256, 0, s>>>(grad, loss);
+    if (cudaGetLastError() != cudaSuccess) return MFC_ECUDA;
+    constexpr int kPerBlock = kGradWarps * kGradGroup;
+    long long blocks = (n + kPerBlock - 1) / kPerBlock;
+    if (blocks > 152) blocks = 152;
+    mlp_grad_kernel<<<(unsigned)blocks, kGradWarps * 32, 0, s>>>(X, Y, n, theta, pos_weight, 1.0f / (float)n, grad,
                                                                  loss);
     return cudaGetLastError() == cudaSuccess ? MFC_OK : MFC_ECUDA;
 }
@@ -306,8 +364,8 @@ extern "C" int mfc_mlp_adam(float* theta, const float* grad, float* m, float* v,
 
 extern "C" int mfc_mlp_forward(const float* X, long long n, const float* theta, float* z, void* cuda_stream) {
     if (!X || !theta || !z || n <= 0) return MFC_EINVAL;
-    long long blocks = (n + 255) / 256;
+    long long blocks = (n + 127) / 128;
     if (blocks > 152LL * 16) blocks = 152LL * 16;
-    mlp_forward_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)cuda_stream>>>(X, n, theta, z);
+    mlp_forward_kernel<<<(unsigned)blocks, 128, 0, (cudaStream_t)cuda_stream>>>(X, n, theta, z);
     return cudaGetLastError() == cudaSuccess ? MFC_OK : MFC_ECUDA;
 }
