@@ -306,8 +306,8 @@ __global__ void conversion_check_kernel(long long n, unsigned long long seed, un
 
 // Self-check of the FP64 form's integer-pipe products K v and quotients x/6
 // against the FP64 instructions, and of its integer-word compares (x > 0,
-// 0 <= x, x < y) against the FP64 compares, and of the integer-pipe quotients
-// against the FP64 division: pseudo-random patterns over every
+// 0 <= x, x < y) against the FP64 compares, and of the integer-pipe quotients,
+// products, squares and square roots against the FP64 instructions: pseudo-random patterns over every
 // exponent, with a share of zeros, subnormals, infinities, NaNs and exponents
 // at the ends of the range where the integer path hands over to the FP64 one;
 // the second compare operand is another such pattern, x itself or x with its
@@ -361,6 +361,17 @@ __global__ void exact_ops_check_kernel(long long n, unsigned long long seed, uns
                            : sel == 10 ? 0.3
                            : sel == 11 ? 0.6
                                        : __longlong_as_double((long long)(((w >> 52) % 600 + 723) << 52 | fn));
+        // products and squares, a zero now and then
+        const double fac = (w & 31u) == 0u ? __longlong_as_double((long long)(z & 0x8000000000000000ULL))
+                                           : __longlong_as_double((long long)(me | (fn & ~((1ULL << cut) - 1)) |
+                                                                              (z & 0x8000000000000000ULL)));
+        bool in = true;
+        const double pr = mul_i(den, fac, in), sr = sq_i(fac, in);
+        // square roots: also of squares and their neighbours
+        const double rt = sel == 12 ? __dmul_rn(den, den) : (sel == 13 ? __dmul_rn(num, num) + den * 0x1p-600 : den);
+        bad += in_range<300>(rt) && __double_as_longlong(sqrt_i(rt)) != __double_as_longlong(sqrt(rt));
+        bad += (__double_as_longlong(pr) != __double_as_longlong(__dmul_rn(den, fac))) +
+               (__double_as_longlong(sr) != __double_as_longlong(__dmul_rn(fac, fac))) + !in;
         bad += mid_range(den) && __double_as_longlong(quot_i(num, rcp_i(den))) != __double_as_longlong(num / den);
     }
     if (bad) atomicAdd(mismatches, bad);

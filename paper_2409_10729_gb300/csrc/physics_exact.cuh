@@ -4,13 +4,14 @@
 // HLLC (Sec. II-B) as physics.cuh, but every formula is evaluated in the
 // textbook order the serial FP64 oracle uses, with one IEEE rounding per
 // operation.  Compiled with -fmad=false (no contraction of a*b+c), the
-// results are bit-identical to that order.  Where several quotients share a
-// denominator, the quotient is formed from a correctly rounded reciprocal
-// y = RN(1/b) and one FMA correction (Markstein's theorem, "Computation of
-// elementary functions on the IBM RISC System/6000", 1990):
-//   q = RN(a y),  r = RN(a - b q) (exact),  a/b rounded = RN(q + r y),
-// which is the correctly rounded a/b for operands without overflow or
-// underflow -- the same bits as a division, at a third of the cost.
+// results are bit-identical to that order.  GB300's FP64 pipe retires two
+// operations per SM and clock, so the quotients, the square roots, WENO5's
+// products and products by small integers are formed from the IEEE 754 fields
+// on the integer pipes -- correctly rounded, hence the same bits.  A division
+// by a width given with its rounded reciprocal y = RN(1/b) takes one FMA
+// correction (Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000", 1990):  q = RN(a y),  r = RN(a - b q) (exact),  RN(q + r y),
+// which is a/b rounded for operands without overflow or underflow.
 #pragma once
 #include "physics.cuh"
 
@@ -117,6 +118,113 @@ __device__ __forceinline__ bool mid_range(double x) {
 
 // a / b out of line, for the rare operands outside that range
 static __device__ __noinline__ double div_any(double a, double b) { return a / b; }
+static __device__ __noinline__ double sqrt_any(double a) { return sqrt(a); }
+
+// ---- correctly rounded products on the integer pipes -------------------------
+// The 106-bit product of two significands (words w3..w0, in [2^104, 2^106))
+// rounded to 53 bits, ties to even: the low 32 + s bits are dropped, their
+// first 32 in f with the rest or-ed into its last bit, and f + 2^31 - 1 + (last
+// kept bit) carries exactly when the kept part has to go up.  e20: sum of the
+// exponent fields less 1024, in place.
+// A product costs about 35 integer instructions with its checks, where the FP64
+// pipe takes 16 clocks a warp: it pays as long as that pipe is the bound and the
+// code stays in the instruction caches.  WENO5's 14 products and squares and
+// HLLC's square roots moved here: FP64 instructions per warp cell 547 -> 440,
+// 256^3 0.464 -> 0.411 ns (the products with everything unrolled 0.454, their
+// loops over indicators and faces kept rolled 0.421).  HLLC's fifty products as
+// well brought 0.400 to 0.469, depending on the block size, and slowed small
+// grids (32^3 0.454 -> 0.478 ms a step): the instruction caches; out of line
+// 0.436.  They stay on the FP64 pipe.
+__device__ __forceinline__ double round_product(unsigned w3, unsigned w2, unsigned w1, unsigned w0, unsigned e20) {
+    const unsigned n = w3 >> 9, s = 20u + n;
+    const unsigned ql = __funnelshift_r(w1, w2, s), qh = __funnelshift_r(w2, w3, s);
+    const unsigned f = __funnelshift_r(w0, w1, s) | min(w0 << (12u - n), 1u);
+    const unsigned up = 0x7fffffffu + (ql & 1u);
+    const unsigned e = e20 + (n << 20);
+    unsigned oh, ol;
+    asm("{\n\t.reg .u32 t;\n\tadd.cc.u32 t, %3, %4;\n\taddc.cc.u32 %1, %2, 0;\n\taddc.u32 %0, %5, %6;\n\t}"
+        : "=r"(oh), "=r"(ol)
+        : "r"(ql), "r"(f), "r"(up), "r"(qh), "r"(e));
+    return __hiloint2double((int)oh, (int)ol);
+}
+
+// |x| within 2^-R .. 2^R
+template <unsigned R>
+__device__ __forceinline__ bool in_range(double x) {
+    return (((unsigned)__double2hiint(x) & 0x7fffffffu) - ((1023u - R) << 20)) < ((2u * R) << 20);
+}
+
+// RN(x^2) for x zero or within 2^-300 .. 2^300 (else ok is cleared)
+__device__ __forceinline__ double sq_i(double x, bool& ok) {
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    const bool zero = ((h << 1) | l) == 0u;
+    ok = ok && (zero || in_range<300>(x));
+    const unsigned m = (h & 0x000fffffu) | 0x00100000u;
+    const unsigned long long t0 = wide(l, l), t1 = wide(l, m << 1) + hi32(t0), t2 = wide(m, m) + hi32(t1);
+    const double r = round_product(hi32(t2), lo32(t2), lo32(t1), lo32(t0), 2u * (h & 0x7ff00000u) - (1024u << 20));
+    return zero ? 0.0 : r;
+}
+
+// RN(a b) for a positive within 2^-300 .. 2^300 and b zero or of a size within
+// that range (else ok is cleared; a is the caller's to check)
+__device__ __forceinline__ double mul_i(double a, double b, bool& ok) {
+    const unsigned ha = (unsigned)__double2hiint(a), la = (unsigned)__double2loint(a);
+    const unsigned hb = (unsigned)__double2hiint(b), lb = (unsigned)__double2loint(b);
+    const bool zero = ((hb << 1) | lb) == 0u;
+    ok = ok && (zero || in_range<300>(b));
+    const unsigned ma = (ha & 0x000fffffu) | 0x00100000u, mb = (hb & 0x000fffffu) | 0x00100000u;
+    const unsigned long long t0 = wide(la, lb), t1 = wide(la, mb) + hi32(t0), t2 = wide(ma, lb) + lo32(t1);
+    const unsigned long long t3 = wide(ma, mb) + (hi32(t1) + hi32(t2));
+    const double r = round_product(hi32(t3), lo32(t3), lo32(t2), lo32(t0),
+                                   (ha & 0x7ff00000u) + (hb & 0x7ff00000u) - (1024u << 20));
+    const unsigned sign = hb & 0x80000000u;
+    return __hiloint2double((int)((zero ? 0u : (unsigned)__double2hiint(r)) | sign),
+                            (int)(zero ? 0u : (unsigned)__double2loint(r)));
+}
+
+// RN(sqrt(a)) for a within 2^-300 .. 2^300.  a = m' 2^(2 k), m' in [2^52, 2^54):
+// the square root's significand is q = RN(sqrt(m' 2^52)).  An FP32 seed I0 2^-23
+// of 1/sqrt(x), x = m' 2^-54, whose residual eps = 1 - x I0^2 2^-46 (below
+// 2^-20, taken from the 101-bit product m' I0^2 without its lowest 32 bits)
+// gives 1/sqrt(x) = I0 (1 + eps/2 + 3/8 eps^2) to 2^-61, then sqrt(x) = x /
+// sqrt(x) to 4 units of 2^-58, low; rounded to 53 bits with 15/32 it is q or
+// q - 1, and N - q^2 - q - 1 >= 0 with N = m' 2^52 (64 bits hold its sign) says
+// which.  A square root of 53-bit integers is never halfway between two.
+__device__ __forceinline__ double sqrt_i(double a) {
+    const unsigned h = (unsigned)__double2hiint(a), l = (unsigned)__double2loint(a);
+    const unsigned odd = ~(h >> 20) & 1u;   // an even exponent field: m doubled
+    const unsigned mh = (h & 0x000fffffu) | 0x00100000u;
+    const unsigned Mh = __funnelshift_l(l, mh, odd), Ml = l << odd;
+    const float x = __uint_as_float((odd ? 0x3f000004u : 0x3e800004u) | ((h & 0x000fffffu) << 3));
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    const unsigned I0 = (__float_as_uint(fmaxf(r, 1.0f)) & 0x007fffffu) | 0x00800000u;
+    const unsigned long long S = wide(I0, I0);
+    const unsigned long long t0 = wide(Ml, hi32(S)) + __umulhi(Ml, lo32(S));
+    const unsigned long long t = wide(Mh, lo32(S)) + t0;
+    unsigned eh = 0u, el = 0u;
+    sub2(eh, el, hi32(t) + Mh * hi32(S), lo32(t));                    // eps 2^68
+    const int em = (int)__funnelshift_r(el, eh, 18);
+    const unsigned long long sq = (unsigned long long)((long long)em * em);   // eps^2 2^100
+    const unsigned long long s3 = wide(hi32(sq), 3u);
+    unsigned ch = (unsigned)((int)eh >> 1), cl = __funnelshift_r(el, eh, 1);
+    add2(ch, cl, hi32(s3) >> 3, __funnelshift_r(lo32(s3), hi32(s3), 3));
+    const unsigned long long T =
+        (unsigned long long)((long long)(int)I0 * (int)ch) + (unsigned long long)__umulhi(I0, cl);
+    const unsigned r0 = lo32(T), r1 = (I0 << 4) + hi32(T);            // 1/sqrt(x) 2^59
+    const unsigned a1 = __funnelshift_l(Ml, Mh, 9), a0 = Ml << 9;
+    const unsigned long long Q = wide(a1, r1) + (__umulhi(a1, r0) + __umulhi(a0, r1) + 15u);   // sqrt(x) 2^58
+    const unsigned ql = __funnelshift_r(lo32(Q), hi32(Q), 5), qh = hi32(Q) >> 5;
+    const unsigned long long q2 = wide(ql, ql) + ql;                  // q^2 + q, low 64 bits
+    const unsigned q2h = hi32(q2) + 2u * (ql * qh) + qh;
+    unsigned dh = Ml << 20, dl = 0u;
+    sub2(dh, dl, q2h, lo32(q2));
+    sub2(dh, dl, 0u, 1u);
+    unsigned oh = ((((h >> 20) - 1075u - odd + 4096u) >> 1) - 2048u + 1048u) << 20, ol = ql;
+    oh += qh;
+    add2(oh, ol, 0u, (~dh) >> 31);
+    return __hiloint2double((int)oh, (int)ol);
+}
 
 // RN(a/b) for any a and b, y = rcp_i(b): signs and a zero numerator are dealt
 // with here, operands outside the middle of the range take the FP64 division.
@@ -295,91 +403,102 @@ __device__ __forceinline__ double div6(double x) {
 // that slides along a pencil can form it once per cell and pass it on.
 __device__ __forceinline__ double curv(double a, double b, double c) {
     const double c13 = 13.0 / 12.0;
-    return c13 * sq(fma2(-2.0, b, a) + c);
+    const double x = fma2(-2.0, b, a) + c;
+    bool ok = true;
+    double t = sq_i(x, ok);
+    t = mul_i(c13, t, ok);
+    if (__builtin_expect(!ok, 0)) t = c13 * sq(x);
+    return t;
 }
 
-// Nonlinear weights of both faces: w[0..2] at i+1/2 (linear weights 0.1, 0.6,
-// 0.3), w[3..5] at i-1/2 (0.3, 0.6, 0.1) from s_k = (eps + beta_k)^2; the
-// quotient 0.6/s1 is the same at both.
-__device__ __forceinline__ void weno5_weights(double s0, double s1, double s2, double* w) {
-    const bool ok = mid_range(s0) && mid_range(s1) && mid_range(s2);
-    const RcpI y0 = rcp_i(s0), y1 = rcp_i(s1), y2 = rcp_i(s2);
-    double a[6] = {quot_i(0.1, y0), quot_i(0.6, y1), quot_i(0.3, y2), quot_i(0.3, y0), 0.0, quot_i(0.1, y2)};
-    a[4] = a[1];
-    const RcpI ym = rcp_i(a[0] + a[1] + a[2]), yp = rcp_i(a[3] + a[4] + a[5]);
-#pragma unroll
+// Both faces' values of WENO5 from x_k, the odd parts' arguments of the three
+// smoothness indicators (beta_k = 1/4 x_k^2 + t_k), and the candidates p (left
+// face) and r (right face): weights a_k = d_k / (eps + beta_k)^2 with d = (0.1,
+// 0.6, 0.3) and (0.3, 0.6, 0.1), omega_k = a_k / sum(a), face value
+// sum omega_k p_k.  Plain FP64 for operands out of the integer forms' range.
+static __device__ __noinline__ void weno5_faces_any(double eps, const double* x, const double* t, const double* p,
+                                                    const double* r, double* out) {
+    double s[3];
+    for (int k = 0; k < 3; ++k) s[k] = sq(eps + fma2(0.25, sq(x[k]), t[k]));
+    const double a0 = 0.1 / s[0], a1 = 0.6 / s[1], a2 = 0.3 / s[2], e0 = 0.3 / s[0], e2 = 0.1 / s[2];
+    const double sm = a0 + a1 + a2, sp = e0 + a1 + e2;
+    out[0] = a0 / sm * p[0] + a1 / sm * p[1] + a2 / sm * p[2];
+    out[1] = e0 / sp * r[0] + a1 / sp * r[1] + e2 / sp * r[2];
+}
+
+__device__ __forceinline__ void weno5_faces(double eps, const double* x, const double* t, const double* p,
+                                            const double* r, double& vm, double& vp) {
+    bool ok = true;
+    // d_k / s_k of both faces (d_1 is the same at both), one indicator a pass,
+    // then the weighted sum, one face a pass: the loops are not unrolled, so
+    // that the code of a reconstruction stays in the instruction caches
+    double x0 = x[0], x1 = x[1], t0 = t[0], t1 = t[1], dm = 0.1, dp = 0.3;
+    double m0 = 0.0, m1 = 0.0, m2 = 0.0, p0 = 0.0, p1 = 0.0, p2 = 0.0;
+#pragma unroll 1
     for (int k = 0; k < 3; ++k) {
-        w[k] = quot_i(a[k], ym);
-        w[3 + k] = quot_i(a[3 + k], yp);
+        const double e = eps + fma2(0.25, sq_i(x0, ok), t0);
+        ok = ok && in_range<150>(e);   // so that every quotient below is normal
+        const RcpI y = rcp_i(sq_i(e, ok));
+        m0 = m1;
+        m1 = m2;
+        m2 = quot_i(dm, y);
+        p0 = p1;
+        p1 = p2;
+        p2 = quot_i(dp, y);
+        x0 = x1;
+        x1 = x[2];
+        t0 = t1;
+        t1 = t[2];
+        dm = k == 0 ? 0.6 : 0.3;
+        dp = k == 0 ? 0.6 : 0.1;
     }
+    double q0 = p[0], q1 = p[1], q2 = p[2], v = 0.0;
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        vm = v;
+        const RcpI y = rcp_i(m0 + m1 + m2);
+        v = mul_i(quot_i(m0, y), q0, ok) + mul_i(quot_i(m1, y), q1, ok) + mul_i(quot_i(m2, y), q2, ok);
+        m0 = p0;
+        m1 = p1;
+        m2 = p2;
+        q0 = r[0];
+        q1 = r[1];
+        q2 = r[2];
+    }
+    vp = v;
     if (__builtin_expect(!ok, 0)) {
-        const double d0 = div_any(0.1, s0), d1 = div_any(0.6, s1), d2 = div_any(0.3, s2);
-        const double e0 = div_any(0.3, s0), e2 = div_any(0.1, s2);
-        const double sm = d0 + d1 + d2, sp = e0 + d1 + e2;
-        w[0] = div_any(d0, sm);
-        w[1] = div_any(d1, sm);
-        w[2] = div_any(d2, sm);
-        w[3] = div_any(e0, sp);
-        w[4] = div_any(d1, sp);
-        w[5] = div_any(e2, sp);
+        double out[2];
+        weno5_faces_any(eps, x, t, p, r, out);
+        vm = out[0];
+        vp = out[1];
     }
 }
 
-// WENO5-JS given the curvature terms t0 = curv(v0, v1, v2), t1 = curv(v1, v2,
-// v3) and t2 = curv(v2, v3, v4) of the three smoothness indicators.
-__device__ __forceinline__ void weno5_t(double eps, double v0, double v1, double v2, double v3, double v4,
-                                        double t0, double t1, double t2, double& vm, double& vp) {
-    // b0 = c13 (v0 - 2 v1 + v2)^2 + 1/4 (v0 - 4 v1 + 3 v2)^2, and likewise b1, b2
-    const double v2x3 = mul_small<3>(v2);
-    double b0 = fma2(0.25, sq(fma2(-4.0, v1, v0) + v2x3), t0);
-    double b1 = fma2(0.25, sq(v1 - v3), t1);
-    double b2 = fma2(0.25, sq(fma2(-4.0, v3, v2x3) + v4), t2);
-    double w[6];
-    weno5_weights(sq(eps + b0), sq(eps + b1), sq(eps + b2), w);
-    const double v2x5 = mul_small<5>(v2), v2x11 = mul_small<11>(v2);
-    double p0 = div6(fma2(2.0, v0, -mul_small<7>(v1)) + v2x11);     // (2 v0 - 7 v1 + 11 v2)/6
-    double p1 = div6(fma2(2.0, v3, -v1 + v2x5));                    // (-v1 + 5 v2 + 2 v3)/6
-    double p2 = div6(fma2(2.0, v2, mul_small<5>(v3)) - v4);         // (2 v2 + 5 v3 - v4)/6
-    vm = w[0] * p0 + w[1] * p1 + w[2] * p2;
-    p0 = div6(fma2(2.0, v2, -v0 + mul_small<5>(v1)));               // (-v0 + 5 v1 + 2 v2)/6
-    p1 = div6(fma2(2.0, v1, v2x5) - v3);                            // (2 v1 + 5 v2 - v3)/6
-    p2 = div6(fma2(2.0, v4, v2x11 - mul_small<7>(v3)));             // (11 v2 - 7 v3 + 2 v4)/6
-    vp = w[3] * p0 + w[4] * p1 + w[5] * p2;
-}
-
-// The right-face candidates of cell i, (-v_{i-2} + 5 v_{i-1} + 2 v_i)/6 and
-// (2 v_{i-1} + 5 v_i - v_{i+1})/6, are the left-face candidates p1 and p2 of
-// cell i-1, formed from the same values in the same order (the same bits):
-// weno5_tc takes them as r0, r1 and returns this cell's p1, p2 for the next.
+// WENO5-JS of cell i from its window, given the curvature terms t0 = curv(v0,
+// v1, v2), t1 = curv(v1, v2, v3) and t2 = curv(v2, v3, v4).  The right-face
+// candidates of cell i, (-v_{i-2} + 5 v_{i-1} + 2 v_i)/6 and (2 v_{i-1} + 5 v_i
+// - v_{i+1})/6, are the left-face candidates p1 and p2 of cell i-1, formed from
+// the same values in the same order (the same bits): weno5_tc takes them as r0,
+// r1 and returns this cell's p1, p2 for the next.
 __device__ __forceinline__ void weno5_tc(double eps, double v0, double v1, double v2, double v3, double v4,
                                          double t0, double t1, double t2, double& r0, double& r1, double& vm,
                                          double& vp) {
-    const double v2x3 = mul_small<3>(v2);
-    double b0 = fma2(0.25, sq(fma2(-4.0, v1, v0) + v2x3), t0);
-    double b1 = fma2(0.25, sq(v1 - v3), t1);
-    double b2 = fma2(0.25, sq(fma2(-4.0, v3, v2x3) + v4), t2);
-    double w[6];
-    weno5_weights(sq(eps + b0), sq(eps + b1), sq(eps + b2), w);
-    const double v2x5 = mul_small<5>(v2), v2x11 = mul_small<11>(v2);
-    double p0 = div6(fma2(2.0, v0, -mul_small<7>(v1)) + v2x11);     // (2 v0 - 7 v1 + 11 v2)/6
-    double p1 = div6(fma2(2.0, v3, -v1 + v2x5));                    // (-v1 + 5 v2 + 2 v3)/6
-    double p2 = div6(fma2(2.0, v2, mul_small<5>(v3)) - v4);         // (2 v2 + 5 v3 - v4)/6
-    vm = w[0] * p0 + w[1] * p1 + w[2] * p2;
-    p0 = div6(fma2(2.0, v4, v2x11 - mul_small<7>(v3)));             // (11 v2 - 7 v3 + 2 v4)/6
-    vp = w[3] * r0 + w[4] * r1 + w[5] * p0;
-    r0 = p1;
-    r1 = p2;
+    const double v2x3 = mul_small<3>(v2), v2x5 = mul_small<5>(v2), v2x11 = mul_small<11>(v2);
+    const double x[3] = {fma2(-4.0, v1, v0) + v2x3, v1 - v3, fma2(-4.0, v3, v2x3) + v4};
+    const double t[3] = {t0, t1, t2};
+    const double p[3] = {div6(fma2(2.0, v0, -mul_small<7>(v1)) + v2x11),     // (2 v0 - 7 v1 + 11 v2)/6
+                         div6(fma2(2.0, v3, -v1 + v2x5)),                    // (-v1 + 5 v2 + 2 v3)/6
+                         div6(fma2(2.0, v2, mul_small<5>(v3)) - v4)};        // (2 v2 + 5 v3 - v4)/6
+    const double r[3] = {r0, r1, div6(fma2(2.0, v4, v2x11 - mul_small<7>(v3)))};   // (11 v2 - 7 v3 + 2 v4)/6
+    weno5_faces(eps, x, t, p, r, vm, vp);
+    r0 = p[1];
+    r1 = p[2];
 }
 
 // The right-face candidates r0, r1 of the cell whose window is v0..v3 (as in weno5_t).
 __device__ __forceinline__ void weno5_right01(double v0, double v1, double v2, double v3, double& r0, double& r1) {
     r0 = div6(fma2(2.0, v2, -v0 + mul_small<5>(v1)));
     r1 = div6(fma2(2.0, v1, mul_small<5>(v2)) - v3);
-}
-
-__device__ __forceinline__ void weno5(double eps, double v0, double v1, double v2, double v3, double v4,
-                                      double& vm, double& vp) {
-    weno5_t(eps, v0, v1, v2, v3, v4, curv(v0, v1, v2), curv(v1, v2, v3), curv(v2, v3, v4), vm, vp);
 }
 
 // WENO3-JS in the reference order: v1..v3 = v_{i-1}..v_{i+1}; weights
@@ -414,17 +533,8 @@ __device__ __forceinline__ void weno3(double eps, double v1, double v2, double v
 }
 
 struct Face {
-    double rho, p, G, Pi, E, c2;
+    double rho, p, G, Pi, E;
 };
-
-template <int NDIM, int NF = 2>
-__device__ __forceinline__ void face_from_prim(const Eos& e, const double* w, Face& s) {
-    using FL = Fields<NDIM, NF>;
-    s.rho = mix_rho<NF>(w);
-    s.p = w[FL::IE];
-    mixture<NF>(e, w + FL::IA, s.G, s.Pi);
-    s.c2 = sound2(s.G, s.Pi, s.rho, s.p);
-}
 
 // Physical flux of side K (primitives w, face state K) normal to DIR; the
 // volume-fraction slots carry alpha_i,K u_n.
@@ -445,16 +555,39 @@ __device__ __forceinline__ void phys_flux(const double* w, const Face& K, double
 // HLLC flux through a face normal to DIR; regions 0<=S_L: F_L, S_L<0<=S*: F*_L,
 // S*<0<=S_R: F*_R, else F_R; the alpha1 slot carries alpha1_K times the
 // region velocity, returned in uf.  Returns true for a non-physical face state.
+// The states are read from wL[f * fs] and wR[f * fs] (shared memory), first
+// side by side for the wave speeds -- one pass of a loop each, so that the
+// instruction caches hold one copy of a side's code -- then the selected side.
 template <int NDIM, int DIR, int NF = 2>
-__device__ __forceinline__ bool hllc(const Eos& e, const double* wL, const double* wR, double* F, double& uf) {
+__device__ __forceinline__ bool hllc(const Eos& e, const double* wL, const double* wR, int fs, double* F, double& uf) {
     using FL = Fields<NDIM, NF>;
-    Face L, R;
-    face_from_prim<NDIM, NF>(e, wL, L);
-    face_from_prim<NDIM, NF>(e, wR, R);
-    bool bad = !gt0(L.rho) || !gt0(R.rho) || !gt0(L.c2) || !gt0(R.c2);
-    double cL = sqrt(L.c2), cR = sqrt(R.c2);
-    double uL = wL[FL::IU + DIR], uR = wR[FL::IU + DIR];
-    const double aL = uL - cL, aR = uR - cR, bL = uL + cL, bR = uR + cR;
+    Face L{}, R{};
+    double aL = 0.0, aR = 0.0, bL = 0.0, bR = 0.0, uL = 0.0, uR = 0.0;
+    bool bad = false;
+    const double* s = wL;
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+        L = R;
+        aL = aR;
+        bL = bR;
+        uL = uR;
+        double rho[NF], al[FL::NA];
+#pragma unroll
+        for (int i = 0; i < NF; ++i) rho[i] = s[i * fs];
+#pragma unroll
+        for (int i = 0; i < FL::NA; ++i) al[i] = s[(FL::IA + i) * fs];
+        R.rho = mix_rho<NF>(rho);
+        R.p = s[FL::IE * fs];
+        mixture<NF>(e, al, R.G, R.Pi);
+        const double c2 = sound2(R.G, R.Pi, R.rho, R.p);
+        bad = bad || !gt0(R.rho) || !gt0(c2);
+        double c = sqrt_i(c2);
+        if (__builtin_expect(!in_range<300>(c2) || !gt0(c2), 0)) c = sqrt_any(c2);
+        uR = s[(FL::IU + DIR) * fs];
+        aR = uR - c;
+        bR = uR + c;
+        s = wR;
+    }
     double SL = less(aL, aR) ? aL : aR;
     double SR = less(bR, bL) ? bL : bR;
     double num = R.p - L.p + L.rho * uL * (SL - uL) - R.rho * uR * (SR - uR);
@@ -462,9 +595,10 @@ __device__ __forceinline__ bool hllc(const Eos& e, const double* wL, const doubl
     double Ss = quot(num, den);
     const bool left = ge0(SL) || ge0(Ss);
     const bool star = left ? !ge0(SL) : ge0(SR);
+    s = left ? wL : wR;
     double w[FL::NEQ];
 #pragma unroll
-    for (int f = 0; f < FL::NEQ; ++f) w[f] = left ? wL[f] : wR[f];
+    for (int f = 0; f < FL::NEQ; ++f) w[f] = s[f * fs];
     Face K;
     K.rho = left ? L.rho : R.rho;
     K.p = left ? L.p : R.p;

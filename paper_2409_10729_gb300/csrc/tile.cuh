@@ -15,14 +15,15 @@
 // enough warps are in flight.  A thread that slides a five-cell window of all
 // fields along its pencil needs 255 registers, 8 warps per SM, and reached 55
 // to 60% of that pipe once the quotients had moved to the integer pipes; one
-// field at a time from shared memory needs 104, 16 warps, and reaches 84%
-// (128^3, ncu: 547 FP64 of 9975 instructions per 32 cells, 0.96 issued per
-// clock).  It also gives small grids parallel work: a thread's serial chain is
+// field at a time from shared memory needs 100, 16 warps, and reaches 80 to 84%
+// (128^3, ncu: 547 FP64 of 9975 instructions per 32 cells and 0.96 issued per
+// clock with WENO's and HLLC's quotients on the integer pipes; 440 and 1.7 with
+// WENO's products and HLLC's square roots there too).  It also gives small grids parallel work: a thread's serial chain is
 // R reconstructions and one flux instead of a segment of whole cells, and a
 // single pencil fills its warps with cells along it.  Measured, sliding window
 // -> tiles: 256^3 droplets 0.557 -> 0.464 ns per cell, equation and RHS;
 // 1024x512 column 6.72 -> 3.36 ms a step; 32^3 RHS 3.9 -> 0.18 ms; 1000-cell
-// tube 2.67 -> 0.041 ms a step.
+// tube 2.67 -> 0.041 ms a step.  (256^3 0.411 now, physics_exact.cuh.)
 #pragma once
 #include <atomic>
 
@@ -218,14 +219,9 @@ __global__ void __launch_bounds__(kTileThreads, MFC_TILE_BLOCKS) tile_kernel(con
     // C: the flux through face j (between cell rows j and j + 1) replaces the
     // right state it was formed from; the region velocity goes to VM[0] row j
     for (int it = threadIdx.x; it < (Jc + 1) << ts.lp; it += T) {
-        double wl[NEQ], wr[NEQ], F[NEQ], uf;
+        double F[NEQ], uf;
         const int o = (it >> ts.lp) * PS + (it & (P - 1));
-#pragma unroll
-        for (int f = 0; f < NEQ; ++f) {
-            wl[f] = VM[f * vf + o];
-            wr[f] = VP[f * vf + o + PS];
-        }
-        const bool fb = exact::hllc<NDIM, DIR, NF>(a.eos, wl, wr, F, uf);
+        const bool fb = exact::hllc<NDIM, DIR, NF>(a.eos, VM + o, VP + o + PS, vf, F, uf);
         bad |= fb && pen0 + (it & (P - 1)) < ts.npen;
 #pragma unroll
         for (int f = 0; f < NEQ; ++f) VP[f * vf + o + PS] = F[f];
