@@ -1,6 +1,6 @@
-// aux.cu -- small kernels around the sweeps: primitive -> conservative
-// conversion, the FP32 working copy of the mixed form, the standalone CFL
-// wave-speed reduction, and the per-step control kernel.  Built with
+// aux.cu -- small kernels around the sweeps: setting a state (primitive ->
+// conservative conversion, FP32 working copy, CFL wave-speed reduction), host
+// copies, and the per-step control kernel.  Built with
 // -fmad=false: the conversion and the wave speed follow the reference
 // operation order bit for bit, so every form starts from the same state.
 #include <stdint.h>
@@ -20,81 +20,77 @@ static unsigned aux_blocks(long long n) {
     return (unsigned)b;
 }
 
-// Primitive (alpha1 rho1, alpha2 rho2, u_k, p, alpha1) -> conservative, in
-// place (Sec. II-A: rho E = Gamma p + Pi + rho |u|^2 / 2), in the reference
-// operation order (this file is built with -fmad=false).
-template <int NDIM, int NF>
-__global__ void prim_to_cons_kernel(double* q, long long nc, Eos e) {
-    using FL = Fields<NDIM, NF>;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc;
-         c += (long long)gridDim.x * blockDim.x) {
-        double w[FL::NEQ], v[FL::NEQ];
-#pragma unroll
-        for (int f = 0; f < FL::NEQ; ++f) w[f] = q[f * nc + c];
-        exact::prim_to_cons<NDIM, NF>(e, w, v);
-#pragma unroll
-        for (int f = 0; f < FL::NEQ; ++f) q[f * nc + c] = v[f];
-    }
-}
-
-// FP32 working copy (conservatives + pressure) of an FP64 state, mixed form.
-template <int NDIM, int NF>
-__global__ void make_mixed_state_kernel(const double* __restrict__ qn, float* __restrict__ s0,
-                                        long long nc, Eos e) {
-    using FL = Fields<NDIM, NF>;
-    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc;
-         c += (long long)gridDim.x * blockDim.x) {
-        double q[FL::NEQ];
-        float q32[FL::NEQ];
-#pragma unroll
-        for (int f = 0; f < FL::NEQ; ++f) {
-            q[f] = qn[f * nc + c];
-            q32[f] = d2f_bits(q[f]);
-            s0[f * nc + c] = q32[f];
-        }
-        s0[FL::NEQ * nc + c] = mixed_pressure<NDIM, NF>(e, q, q32);
-    }
-}
-
-// S = max over cells of sum_d (|u_d| + c)/dx_d of an FP64 state, in the
-// reference operation order.
-template <int NDIM, int NF>
-__global__ void wavespeed_kernel(const double* __restrict__ q, long long nc, Eos e, double dx0, double dx1,
-                                 double dx2, double rdx0, double rdx1, double rdx2, DevCtrl* ctrl, int n0, int n1,
-                                 Geom3 g) {
+// Sets a state in one pass over the cells: the conservative state qn from src
+// (conservative, or primitive with PRIM: rho E = Gamma p + Pi + rho |u|^2 / 2,
+// Sec. II-A), the FP32 working copy s0 with the pressure (FP32 forms, MIXED),
+// and S = max over cells of sum_d (|u_d| + c)/dx_d, all in the reference
+// operation order.  src may be qn itself; with neither PRIM nor MIXED nor
+// another src it only reduces S.  A cell is read and written once: conversion,
+// copies and wave speed as kernels of their own moved 2.5 times the bytes and
+// formed the mixture rules three times.  The FP64 pipe bounds it, so its
+// products are integer ones too (exact::MulInt).  Measured, 512^3 mixed, the
+// call: 27.8 ms as four kernels with FP64 divisions, 14.1 fused with integer
+// quotients and roots (FP64 pipe 84% busy), 12.8 with integer products at three
+// blocks per SM (128 registers, two blocks: 18.6).
+template <int NDIM, int NF, bool PRIM, bool MIXED>
+__global__ void __launch_bounds__(kAuxThreads, 3)
+set_state_kernel(const double* src, double* qn, float* __restrict__ s0, long long nc, Eos e, double dx0, double dx1,
+                 double dx2, double rdx0, double rdx1, double rdx2, DevCtrl* ctrl, int n0, int n1, Geom3 g) {
     using FL = Fields<NDIM, NF>;
     double dx[3] = {dx0, dx1, dx2};
     double rdx[3] = {rdx0, rdx1, rdx2};
     double smax = 0.0;
     bool bad = false;
-    long long stride = (long long)gridDim.x * blockDim.x;
-    long long start = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    // every thread of a warp runs the same number of iterations so that the
-    // warp reduction below sees all 32 lanes
-    long long iters = (nc + stride - 1) / stride;
+    const bool store = PRIM || src != qn;
     // uniform over the launch: only a non-uniform grid needs the cell's
     // coordinates (64-bit divisions, kept off the uniform-grid path)
     const bool nu = g.cw[0] || g.cw[1] || g.cw[2];
-    for (long long it = 0; it < iters; ++it) {
-        long long c = start + it * stride;
-        if (c < nc) {
-            double v[FL::NEQ];
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc; c += stride) {
+        double v[FL::NEQ], q[FL::NEQ];
 #pragma unroll
-            for (int f = 0; f < FL::NEQ; ++f) v[f] = __ldg(q + f * nc + c);
-            if (nu) {   // non-uniform directions: the cell's own width
-                const long long ci[3] = {c % n0, (c / n0) % n1, c / ((long long)n0 * n1)};
+        for (int f = 0; f < FL::NEQ; ++f) v[f] = src[f * nc + c];
+        bool ok = true;
+        const exact::MulInt mul{ok};
+        if constexpr (PRIM) {
+            exact::prim_to_cons<NDIM, NF>(e, v, q, mul);
+            if (__builtin_expect(!ok, 0)) exact::prim_to_cons<NDIM, NF>(e, v, q);
+        } else {
 #pragma unroll
-                for (int d = 0; d < NDIM; ++d)
-                    if (g.cw[d]) {
-                        dx[d] = __ldg(g.cw[d] + ci[d]);
-                        rdx[d] = __ldg(g.crw[d] + ci[d]);
-                    }
-            }
-            double s = exact::cell_wavespeed<NDIM, NF>(e, v, dx, rdx, bad);
-            smax = s > smax ? s : smax;
+            for (int f = 0; f < FL::NEQ; ++f) q[f] = v[f];
         }
+        if (store) {
+#pragma unroll
+            for (int f = 0; f < FL::NEQ; ++f) qn[f * nc + c] = q[f];
+        }
+        if constexpr (MIXED) {
+            float q32[FL::NEQ];
+#pragma unroll
+            for (int f = 0; f < FL::NEQ; ++f) {
+                q32[f] = d2f_bits(q[f]);
+                s0[f * nc + c] = q32[f];
+            }
+            s0[FL::NEQ * nc + c] = mixed_pressure<NDIM, NF>(e, q, q32);
+        }
+        if (nu) {   // non-uniform directions: the cell's own width
+            const long long ci[3] = {c % n0, (c / n0) % n1, c / ((long long)n0 * n1)};
+#pragma unroll
+            for (int d = 0; d < NDIM; ++d)
+                if (g.cw[d]) {
+                    dx[d] = __ldg(g.cw[d] + ci[d]);
+                    rdx[d] = __ldg(g.crw[d] + ci[d]);
+                }
+        }
+        bool cbad = false;
+        double s = exact::cell_wavespeed<NDIM, NF>(e, q, dx, rdx, cbad, mul);
+        if (__builtin_expect(!ok, 0)) {   // operands out of the integer products' range
+            cbad = false;
+            s = exact::cell_wavespeed<NDIM, NF>(e, q, dx, rdx, cbad);
+        }
+        bad |= cbad;
+        smax = s > smax ? s : smax;
     }
-    double m = warp_max(smax);
+    const double m = warp_max(smax);
     if ((threadIdx.x & 31) == 0 && m > 0.0)
         atomicMax(&ctrl->S_bits, (unsigned long long)__double_as_longlong(m));
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&ctrl->status, 1u);
@@ -110,12 +106,6 @@ __global__ void step_begin_kernel(DevCtrl* ctrl) {
     ctrl->dt = dt;
     ctrl->t += dt;
     ctrl->S_bits = 0ULL;
-}
-
-__global__ void f32_to_f64_kernel(const float* __restrict__ src, double* __restrict__ dst, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        dst[i] = double(src[i]);
 }
 
 // Calls f.template operator()<NDIM, NF>() for the runtime ndim and fluid count.
@@ -138,26 +128,9 @@ cudaError_t dispatch_nd_nf(int ndim, int nf, Fn&& f) {
     }
 }
 
-cudaError_t launch_prim_to_cons(int ndim, double* q, long long nc, const Eos& e, cudaStream_t s) {
-    unsigned g = aux_blocks(nc);
-    return dispatch_nd_nf(ndim, e.nf, [&]<int ND, int NF>() {
-        prim_to_cons_kernel<ND, NF><<<g, kAuxThreads, 0, s>>>(q, nc, e);
-        return cudaGetLastError();
-    });
-}
-
-cudaError_t launch_make_mixed_state(int ndim, const double* qn, float* s0, long long nc, const Eos& e,
-                                    cudaStream_t s) {
-    unsigned g = aux_blocks(nc);
-    return dispatch_nd_nf(ndim, e.nf, [&]<int ND, int NF>() {
-        make_mixed_state_kernel<ND, NF><<<g, kAuxThreads, 0, s>>>(qn, s0, nc, e);
-        return cudaGetLastError();
-    });
-}
-
-cudaError_t launch_wavespeed(int ndim, const double* q, const int* n, const double* const* cw,
-                             const double* const* crw, long long nc, const double* dx, const double* rdx,
-                             const Eos& e, DevCtrl* ctrl, cudaStream_t s) {
+cudaError_t launch_set_state(int ndim, const double* src, bool prim, double* qn, float* s0, const int* n,
+                             const double* const* cw, const double* const* crw, long long nc, const double* dx,
+                             const double* rdx, const Eos& e, DevCtrl* ctrl, cudaStream_t s) {
     cudaError_t err = cudaMemsetAsync(&ctrl->S_bits, 0, sizeof(unsigned long long), s);
     if (err != cudaSuccess) return err;
     Geom3 g3;
@@ -165,21 +138,20 @@ cudaError_t launch_wavespeed(int ndim, const double* q, const int* n, const doub
         g3.cw[d] = cw ? cw[d] : nullptr;
         g3.crw[d] = crw ? crw[d] : nullptr;
     }
-    unsigned g = aux_blocks(nc);
+    const unsigned g = aux_blocks(nc);
     return dispatch_nd_nf(ndim, e.nf, [&]<int ND, int NF>() {
-        wavespeed_kernel<ND, NF><<<g, kAuxThreads, 0, s>>>(q, nc, e, dx[0], dx[1], dx[2], rdx[0], rdx[1], rdx[2],
-                                                          ctrl, n[0], n[1], g3);
-        return cudaGetLastError();
+        auto go = [&](auto kernel) {
+            kernel<<<g, kAuxThreads, 0, s>>>(src, qn, s0, nc, e, dx[0], dx[1], dx[2], rdx[0], rdx[1], rdx[2], ctrl,
+                                             n[0], n[1], g3);
+            return cudaGetLastError();
+        };
+        if (prim) return s0 ? go(set_state_kernel<ND, NF, true, true>) : go(set_state_kernel<ND, NF, true, false>);
+        return s0 ? go(set_state_kernel<ND, NF, false, true>) : go(set_state_kernel<ND, NF, false, false>);
     });
 }
 
 cudaError_t launch_step_begin(DevCtrl* ctrl, cudaStream_t s) {
     step_begin_kernel<<<1, 1, 0, s>>>(ctrl);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_f32_to_f64(const float* src, double* dst, long long n, cudaStream_t s) {
-    f32_to_f64_kernel<<<aux_blocks(n), kAuxThreads, 0, s>>>(src, dst, n);
     return cudaGetLastError();
 }
 

@@ -383,37 +383,30 @@ static int ensure_graph(mfc_ctx* ctx) {
     return MFC_OK;
 }
 
-static int after_state_change(mfc_ctx* ctx) {
-    if (fp32_state(ctx))
-        CK(launch_make_mixed_state(ctx->ndim, ctx->qn, ctx->s0, ctx->ncell, ctx->eos, ctx->stream));
-    CK(launch_wavespeed(ctx->ndim, ctx->qn, ctx->n, ctx->gw, ctx->grw, ctx->ncell, ctx->dx, ctx->rdx, ctx->eos,
-                        ctx->ctrl, ctx->stream));
+// Launches the state set-up from src (q^n itself to reduce S only).
+static cudaError_t set_state_from(mfc_ctx* ctx, const double* src, bool prim, float* s0) {
+    return launch_set_state(ctx->ndim, src, prim, ctx->qn, s0, ctx->n, ctx->gw, ctx->grw, ctx->ncell, ctx->dx,
+                            ctx->rdx, ctx->eos, ctx->ctrl, ctx->stream);
+}
+
+static int set_state_impl(mfc_ctx* ctx, const double* src, int on_device, bool prim) {
+    if (!ctx || !src) return MFC_EINVAL;
+    if (!on_device) {
+        CK(host_copy(ctx->qn, src, (size_t)ctx->ncell * ctx->neq * sizeof(double), true, ctx->stream));
+        src = ctx->qn;
+    }
+    CK(set_state_from(ctx, src, prim, fp32_state(ctx) ? ctx->s0 : NULL));
     ctx->have_state = true;
+    if (!on_device) CK(cudaStreamSynchronize(ctx->stream));
     return MFC_OK;
 }
 
-
 extern "C" int mfc_set_state(mfc_ctx* ctx, const double* q, int on_device) {
-    if (!ctx || !q) return MFC_EINVAL;
-    size_t bytes = (size_t)ctx->ncell * ctx->neq * sizeof(double);
-    CK(on_device ? cudaMemcpyAsync(ctx->qn, q, bytes, cudaMemcpyDeviceToDevice, ctx->stream)
-                 : host_copy(ctx->qn, q, bytes, true, ctx->stream));
-    int st = after_state_change(ctx);
-    if (st) return st;
-    if (!on_device) CK(cudaStreamSynchronize(ctx->stream));
-    return MFC_OK;
+    return set_state_impl(ctx, q, on_device, false);
 }
 
 extern "C" int mfc_set_state_prim(mfc_ctx* ctx, const double* w, int on_device) {
-    if (!ctx || !w) return MFC_EINVAL;
-    size_t bytes = (size_t)ctx->ncell * ctx->neq * sizeof(double);
-    CK(on_device ? cudaMemcpyAsync(ctx->qn, w, bytes, cudaMemcpyDeviceToDevice, ctx->stream)
-                 : host_copy(ctx->qn, w, bytes, true, ctx->stream));
-    CK(launch_prim_to_cons(ctx->ndim, ctx->qn, ctx->ncell, ctx->eos, ctx->stream));
-    int st = after_state_change(ctx);
-    if (st) return st;
-    if (!on_device) CK(cudaStreamSynchronize(ctx->stream));
-    return MFC_OK;
+    return set_state_impl(ctx, w, on_device, true);
 }
 
 extern "C" int mfc_get_state(mfc_ctx* ctx, double* q, int on_device) {
@@ -513,8 +506,7 @@ extern "C" int mfc_max_wavespeed(mfc_ctx* ctx, double* s) {
     if (!ctx->have_state) return MFC_ESTATE;
     int st = write_ctrl_params(ctx, 0.0, 0.0);
     if (st) return st;
-    CK(launch_wavespeed(ctx->ndim, ctx->qn, ctx->n, ctx->gw, ctx->grw, ctx->ncell, ctx->dx, ctx->rdx, ctx->eos,
-                        ctx->ctrl, ctx->stream));
+    CK(set_state_from(ctx, ctx->qn, false, NULL));
     st = read_ctrl(ctx);
     if (st) return st;
     unsigned long long bits = ctx->ctrl_h->S_bits;
@@ -619,8 +611,7 @@ extern "C" int mfc_set_grid(mfc_ctx* ctx, int dir, const double* edges) {
     ctx->grw[dir] = nrw;
     ctx->grw32[dir] = nrw32;
     if (ctx->have_state) {
-        CK(launch_wavespeed(ctx->ndim, ctx->qn, ctx->n, ctx->gw, ctx->grw, ctx->ncell, ctx->dx, ctx->rdx, ctx->eos,
-                            ctx->ctrl, ctx->stream));
+        CK(set_state_from(ctx, ctx->qn, false, NULL));
         CK(cudaStreamSynchronize(ctx->stream));
     }
     return MFC_OK;

@@ -151,14 +151,12 @@ cudaError_t launch_gate_samples(int ndim, const double* q, const int* n, const i
                                 double eps, float tau, float* X, float* Y, cudaStream_t s);
 
 // auxiliary kernels (aux.cu)
-cudaError_t launch_prim_to_cons(int ndim, double* q, long long ncell, const Eos& e, cudaStream_t s);
-cudaError_t launch_make_mixed_state(int ndim, const double* qn, float* s0, long long ncell,
-                                    const Eos& e, cudaStream_t s);
-cudaError_t launch_wavespeed(int ndim, const double* q, const int* n, const double* const* cw,
-                             const double* const* crw, long long ncell, const double* dx,
+// state set-up: qn from src (primitive with prim; src may be qn), the FP32 copy
+// s0 of the FP32 forms (or null), and S into ctrl
+cudaError_t launch_set_state(int ndim, const double* src, bool prim, double* qn, float* s0, const int* n,
+                             const double* const* cw, const double* const* crw, long long nc, const double* dx,
                              const double* rdx, const Eos& e, DevCtrl* ctrl, cudaStream_t s);
 cudaError_t launch_step_begin(DevCtrl* ctrl, cudaStream_t s);
-cudaError_t launch_f32_to_f64(const float* src, double* dst, long long count, cudaStream_t s);
 // Host <-> device copy of a state-sized array.  When the host side is
 // page-locked and mapped into the device's address space (unified
 // addressing), and both addresses and the size are multiples of 16 bytes, the

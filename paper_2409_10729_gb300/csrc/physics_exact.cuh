@@ -182,6 +182,28 @@ __device__ __forceinline__ double mul_i(double a, double b, bool& ok) {
                             (int)(zero ? 0u : (unsigned)__double2loint(r)));
 }
 
+// RN(a b) for a and b each zero or within 2^-300 .. 2^300 in size (else ok is cleared)
+__device__ __forceinline__ double mul_s(double a, double b, bool& ok) {
+    const unsigned ha = (unsigned)__double2hiint(a), la = (unsigned)__double2loint(a);
+    const bool zero = ((ha << 1) | la) == 0u;
+    ok = ok && (zero || in_range<300>(a));
+    const double r = mul_i(a, b, ok);   // the sign of b
+    const unsigned h = (unsigned)__double2hiint(r);
+    return __hiloint2double((int)((zero ? h & 0x80000000u : h) ^ (ha & 0x80000000u)),
+                            zero ? 0 : __double2loint(r));
+}
+
+// How the EOS functions below form their products: on the FP64 pipe, or on the
+// integer pipes (the same bits; ok is cleared when an operand was out of range
+// and the results do not count).
+struct MulFp {
+    __device__ __forceinline__ double operator()(double a, double b) const { return a * b; }
+};
+struct MulInt {
+    bool& ok;
+    __device__ __forceinline__ double operator()(double a, double b) const { return mul_s(a, b, ok); }
+};
+
 // RN(sqrt(a)) for a within 2^-300 .. 2^300.  a = m' 2^(2 k), m' in [2^52, 2^54):
 // the square root's significand is q = RN(sqrt(m' 2^52)).  An FP32 seed I0 2^-23
 // of 1/sqrt(x), x = m' 2^-54, whose residual eps = 1 - x I0^2 2^-46 (below
@@ -226,6 +248,12 @@ __device__ __forceinline__ double sqrt_i(double a) {
     return __hiloint2double((int)oh, (int)ol);
 }
 
+// RN(sqrt(a)) for any a
+__device__ __forceinline__ double sqrt_p(double a) {
+    const double r = sqrt_i(a);
+    return __builtin_expect(in_range<300>(a) && gt0(a), 1) ? r : sqrt_any(a);
+}
+
 // RN(a/b) for any a and b, y = rcp_i(b): signs and a zero numerator are dealt
 // with here, operands outside the middle of the range take the FP64 division.
 __device__ __forceinline__ double quot(double a, double b, const RcpI& y) {
@@ -248,19 +276,19 @@ __device__ __forceinline__ double sq(double x) { return x * x; }
 // Gamma = sum_i alpha_i g_i, Pi = sum_i alpha_i P_i over the NF fluids, the
 // carried fractions a[0..NF-2] first and alpha_N = 1 - a[0] - ... - a[NF-2]
 // last (two fluids: a1 g1 + (1 - a1) g2).
-template <int NF>
-__device__ __forceinline__ void mixture(const Eos& e, const double* a, double& G, double& Pi) {
+template <int NF, typename M>
+__device__ __forceinline__ void mixture(const M& mul, const Eos& e, const double* a, double& G, double& Pi) {
     double aN = 1.0 - a[0];
 #pragma unroll
     for (int i = 1; i < NF - 1; ++i) aN = aN - a[i];
-    double sg = a[0] * e.g[0], sp = a[0] * e.P[0];
+    double sg = mul(a[0], e.g[0]), sp = mul(a[0], e.P[0]);
 #pragma unroll
     for (int i = 1; i < NF - 1; ++i) {
-        sg = sg + a[i] * e.g[i];
-        sp = sp + a[i] * e.P[i];
+        sg = sg + mul(a[i], e.g[i]);
+        sp = sp + mul(a[i], e.P[i]);
     }
-    G = sg + aN * e.g[NF - 1];
-    Pi = sp + aN * e.P[NF - 1];
+    G = sg + mul(aN, e.g[NF - 1]);
+    Pi = sp + mul(aN, e.P[NF - 1]);
 }
 
 template <int NF>
@@ -273,26 +301,26 @@ __device__ __forceinline__ double mix_rho(const double* q) {
 
 // 0.5 rho |u|^2 in the oracle's order, whose sum starts from 0.0: 0.0 + u_0^2
 // is u_0^2 itself (a square is never -0), so the sum starts there.
-template <int NDIM>
-__device__ __forceinline__ double kinetic(double rho, const double* u) {
-    double s = u[0] * u[0];
+template <int NDIM, typename M>
+__device__ __forceinline__ double kinetic(const M& mul, double rho, const double* u) {
+    double s = mul(u[0], u[0]);
 #pragma unroll
-    for (int k = 1; k < NDIM; ++k) s = s + u[k] * u[k];
-    return 0.5 * rho * s;
+    for (int k = 1; k < NDIM; ++k) s = s + mul(u[k], u[k]);
+    return mul(0.5 * rho, s);
 }
 
 // Conservative -> primitive (u_k = rho u_k / rho, p = (rho E - ke - Pi)/Gamma).
-template <int NDIM, int NF = 2>
-__device__ __forceinline__ void cons_to_prim(const Eos& e, const double* q, double* w) {
+template <int NDIM, int NF = 2, typename M = MulFp>
+__device__ __forceinline__ void cons_to_prim(const Eos& e, const double* q, double* w, const M& mul = M()) {
     using FL = Fields<NDIM, NF>;
     double rho = mix_rho<NF>(q);
     const RcpI y = rcp_i(rho);
     double u[NDIM];
 #pragma unroll
     for (int k = 0; k < NDIM; ++k) u[k] = quot(q[FL::IU + k], rho, y);
-    double ke = kinetic<NDIM>(rho, u);
+    double ke = kinetic<NDIM>(mul, rho, u);
     double G, Pi;
-    mixture<NF>(e, q + FL::IA, G, Pi);
+    mixture<NF>(mul, e, q + FL::IA, G, Pi);
     double p = quot(q[FL::IE] - ke - Pi, G);
 #pragma unroll
     for (int i = 0; i < NF; ++i) w[i] = q[i];
@@ -304,27 +332,28 @@ __device__ __forceinline__ void cons_to_prim(const Eos& e, const double* q, doub
 }
 
 // Primitive -> conservative (rho E = Gamma p + Pi + ke).
-template <int NDIM, int NF = 2>
-__device__ __forceinline__ void prim_to_cons(const Eos& e, const double* w, double* q) {
+template <int NDIM, int NF = 2, typename M = MulFp>
+__device__ __forceinline__ void prim_to_cons(const Eos& e, const double* w, double* q, const M& mul = M()) {
     using FL = Fields<NDIM, NF>;
     double rho = mix_rho<NF>(w);
     double u[NDIM];
 #pragma unroll
     for (int k = 0; k < NDIM; ++k) u[k] = w[FL::IU + k];
-    double ke = kinetic<NDIM>(rho, u);
+    double ke = kinetic<NDIM>(mul, rho, u);
     double G, Pi;
-    mixture<NF>(e, w + FL::IA, G, Pi);
+    mixture<NF>(mul, e, w + FL::IA, G, Pi);
 #pragma unroll
     for (int i = 0; i < NF; ++i) q[i] = w[i];
 #pragma unroll
-    for (int k = 0; k < NDIM; ++k) q[FL::IU + k] = rho * u[k];
-    q[FL::IE] = G * w[FL::IE] + Pi + ke;
+    for (int k = 0; k < NDIM; ++k) q[FL::IU + k] = mul(rho, u[k]);
+    q[FL::IE] = mul(G, w[FL::IE]) + Pi + ke;
 #pragma unroll
     for (int i = 0; i < FL::NA; ++i) q[FL::IA + i] = w[FL::IA + i];
 }
 
-__device__ __forceinline__ double sound2(double G, double Pi, double rho, double p) {
-    return quot((G + 1.0) * p + Pi, G * rho);
+template <typename M>
+__device__ __forceinline__ double sound2(const M& mul, double G, double Pi, double rho, double p) {
+    return quot(mul(G + 1.0, p) + Pi, mul(G, rho));
 }
 
 // WENO5-JS: left-biased value at i+1/2 and right-biased value at i-1/2 from
@@ -578,11 +607,10 @@ __device__ __forceinline__ bool hllc(const Eos& e, const double* wL, const doubl
         for (int i = 0; i < FL::NA; ++i) al[i] = s[(FL::IA + i) * fs];
         R.rho = mix_rho<NF>(rho);
         R.p = s[FL::IE * fs];
-        mixture<NF>(e, al, R.G, R.Pi);
-        const double c2 = sound2(R.G, R.Pi, R.rho, R.p);
+        mixture<NF>(MulFp(), e, al, R.G, R.Pi);
+        const double c2 = sound2(MulFp(), R.G, R.Pi, R.rho, R.p);
         bad = bad || !gt0(R.rho) || !gt0(c2);
-        double c = sqrt_i(c2);
-        if (__builtin_expect(!in_range<300>(c2) || !gt0(c2), 0)) c = sqrt_any(c2);
+        const double c = sqrt_p(c2);
         uR = s[(FL::IU + DIR) * fs];
         aR = uR - c;
         bR = uR + c;
@@ -604,7 +632,7 @@ __device__ __forceinline__ bool hllc(const Eos& e, const double* wL, const doubl
     K.p = left ? L.p : R.p;
     K.G = left ? L.G : R.G;
     K.Pi = left ? L.Pi : R.Pi;
-    K.E = K.G * K.p + K.Pi + kinetic<NDIM>(K.rho, w + FL::IU);   // of the selected side only
+    K.E = K.G * K.p + K.Pi + kinetic<NDIM>(MulFp(), K.rho, w + FL::IU);   // of the selected side only
     double SK = left ? SL : SR;
     double un = w[FL::IU + DIR];
     phys_flux<NDIM, DIR, NF>(w, K, F);
@@ -628,18 +656,18 @@ __device__ __forceinline__ bool hllc(const Eos& e, const double* wL, const doubl
 }
 
 // S contribution of one cell: sum_d (|u_d| + c)/dx_d, from the conservative state.
-template <int NDIM, int NF = 2>
+template <int NDIM, int NF = 2, typename M = MulFp>
 __device__ __forceinline__ double cell_wavespeed(const Eos& e, const double* q, const double* dx,
-                                                 const double* rdx, bool& bad) {
+                                                 const double* rdx, bool& bad, const M& mul = M()) {
     using FL = Fields<NDIM, NF>;
     double w[FL::NEQ];
-    cons_to_prim<NDIM, NF>(e, q, w);
+    cons_to_prim<NDIM, NF>(e, q, w, mul);
     double rho = mix_rho<NF>(w);
     double G, Pi;
-    mixture<NF>(e, w + FL::IA, G, Pi);
-    double c2 = sound2(G, Pi, rho, w[FL::IE]);
+    mixture<NF>(mul, e, w + FL::IA, G, Pi);
+    double c2 = sound2(mul, G, Pi, rho, w[FL::IE]);
     bad |= !gt0(mix_rho<NF>(q)) || !gt0(rho) || !gt0(c2);
-    double cs = sqrt(c2);
+    const double cs = sqrt_p(c2);
     double s = 0.0;
 #pragma unroll
     for (int d = 0; d < NDIM; ++d) s = s + div_rcp(fabs(w[FL::IU + d]) + cs, dx[d], rdx[d]);
