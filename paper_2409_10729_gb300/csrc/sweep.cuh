@@ -407,18 +407,21 @@ __device__ __forceinline__ void gate_logits(const GateSmem& g, uint4* tile, cons
 // Relative round-off floor of the gate's flat test (MFC_GATE_FLOOR).
 constexpr float kGateFloor32 = (float)MFC_GATE_FLOOR;
 
-// Normalised sensor stencil: x_k = (v_k - v_2) / max_j |v_j - v_2|.  Returns
-// false, with x = 0, when the stencil is flat -- max_j |v_j - v_2| <= floor
-// |v_2| -- and counts as smooth without the network.
-__device__ __forceinline__ bool gate_input(const float* v, float* x) {
-    float m = 0.f;
+// Largest difference max_k |v_k - v_2| of a sensor stencil; live when it is above
+// floor |v_2|.  A stencil that is not live is flat and counts as smooth without
+// the network.
+__device__ __forceinline__ bool gate_live(const float* v, float& m) {
+    m = 0.f;
 #pragma unroll
     for (int k = 0; k < 5; ++k) m = fmaxf(m, fabsf(v[k] - v[2]));
-    const bool live = m > kGateFloor32 * fabsf(v[2]);
+    return m > kGateFloor32 * fabsf(v[2]);
+}
+
+// The network's input x_k = (v_k - v_2) / m, 0 for a flat stencil.
+__device__ __forceinline__ void gate_input(const float* v, float m, bool live, float* x) {
     const float r = live ? __frcp_rn(m) : 0.f;
 #pragma unroll
     for (int k = 0; k < 5; ++k) x[k] = (v[k] - v[2]) * r;
-    return live;
 }
 
 // Linear-weight (fifth-order upwind) face values of cell i: the WENO5
@@ -427,6 +430,19 @@ __device__ __forceinline__ void linear5(float v0, float v1, float v2, float v3, 
     float d1 = v1 - v0, d2 = v2 - v1, d3 = v3 - v2, d4 = v4 - v3;
     vm = v2 + (0.1f * (5.f * d2 - 2.f * d1) + 0.6f * (d2 + 2.f * d3) + 0.3f * (4.f * d3 - d4)) * (1.f / 6.f);
     vp = v2 + (0.3f * (d1 - 4.f * d2) - 0.6f * (2.f * d2 + d3) + 0.1f * (2.f * d4 - 5.f * d3)) * (1.f / 6.f);
+}
+
+// The same for two fields, packed, rounded as the compiler contracts linear5.
+__device__ __forceinline__ void linear5_pair(F2 v0, F2 v1, F2 v2, F2 v3, F2 v4, F2& vm, F2& vp) {
+    const F2 d1 = sub(v1, v0), d2 = sub(v2, v1), d3 = sub(v3, v2), d4 = sub(v4, v3);
+    const F2 a = fma2x(f2(5.f), d2, mul(f2(-2.f), d1)), b = fma2x(f2(2.f), d3, d2);
+    const F2 c = fma2x(f2(4.f), d3, mul(f2(-1.f), d4));
+    const F2 s = fma2x(f2(0.1f), a, mul(f2(0.6f), b));
+    vm = fma2x(fma2x(f2(0.3f), c, s), f2(1.f / 6.f), v2);
+    const F2 e = fma2x(f2(-4.f), d2, d1), g = fma2x(f2(2.f), d2, d3);
+    const F2 h = fma2x(f2(-5.f), d3, mul(f2(2.f), d4));
+    const F2 t = fma2x(f2(0.3f), e, mul(f2(-0.6f), g));
+    vp = fma2x(fma2x(f2(0.1f), h, t), f2(1.f / 6.f), v2);
 }
 
 // A reconstructed face state is usable when rho > 0, 0 <= alpha1 <= 1 and
@@ -476,20 +492,22 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
 // Minimum resident blocks for the register allocator, in blocks of the
 // sweep's own size (x sweeps run one-warp blocks, each with its own output
 // tile in static shared memory).
-template <int FORM, int MODE, int DIR, int NF = 2>
+template <int FORM, int MODE, int DIR, int NF = 2, int NDIM = 3>
 constexpr int sweep_min_blocks() {
     if (NF > 2) return 1;   // more fields per cell: no register cap (the two-fluid caps spill)
     constexpr int per128 = FORM == FORM_MIXED   ? (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_MIXED_RK
-                                                   : DIR == 0         ? MFC_MIN_BLOCKS_MIXED_X
+                                                   : DIR == 0         ? (NDIM == 2 ? MFC_MIN_BLOCKS_MIXED_X2 : MFC_MIN_BLOCKS_MIXED_X)
                                                                       : MFC_MIN_BLOCKS_MIXED)
-                                                : (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_GATED_RK : MFC_MIN_BLOCKS_GATED);
+                                                : (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_GATED_RK
+                                                   : DIR == 0       ? MFC_MIN_BLOCKS_GATED_X
+                                                                    : MFC_MIN_BLOCKS_GATED);
     return per128 * 128 / sweep_threads(DIR);
 }
 
 // NU: some direction of the grid is non-uniform (tables, per-cell widths);
 // the uniform-grid kernels carry none of that code.
 template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF>
-__global__ void __launch_bounds__(sweep_threads(DIR), sweep_min_blocks<FORM, MODE, DIR, NF>())
+__global__ void __launch_bounds__(sweep_threads(DIR), sweep_min_blocks<FORM, MODE, DIR, NF, NDIM>())
 sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
     using R = FormReal<FORM>;
     constexpr bool GATED = FORM == FORM_GATED;
@@ -718,6 +736,8 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
         // mixed form, x sweep: the first differences d1..d3 and curvature parts C0, C1
         // of the window's centre cell, carried along the pencil (weno5_dc); the y and
         // z sweeps, register-capped for occupancy, lose more to spills than it saves
+        // reconstruct two fields at a time (packed FP32 pairs, physics.cuh)
+        constexpr bool PACK = !NU;
         constexpr bool DCARRY = FORM == FORM_MIXED && !NU && DIR == 0 && MFC_DIFF_CARRY;
         float Dd1[DCARRY ? NEQ : 1], Dd2[DCARRY ? NEQ : 1], Dd3[DCARRY ? NEQ : 1];
         float Cc0[DCARRY ? NEQ : 1], Cc1[DCARRY ? NEQ : 1];
@@ -781,14 +801,28 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
                     sr[k] = W[k][0] + W[k][1];
                     sp[k] = W[k][IE];
                 }
-                const bool live_r = gate_input(sr, xr), live_p = gate_input(sp, xp);
+                float mr, mp;
+                const bool live_r = gate_live(sr, mr), live_p = gate_live(sp, mp);
                 const bool warp_flat = !__any_sync(0xffffffffu, live_r || live_p);
-                if (!warp_flat)
+                if (!warp_flat) {
+                    gate_input(sr, mr, live_r, xr);
+                    gate_input(sp, mp, live_p, xp);
                     gate_logits(gsm[0], gtile + (threadIdx.x >> 5) * 128, xr, xp, live_r, live_p, true, zr, zp);
+                }
                 const bool smooth = (!live_r || zr < 0.f) && (!live_p || zp < 0.f);
                 if (smooth) {
 #pragma unroll
-                    for (int f = 0; f < NEQ; ++f) linear5(W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], vm[f], vp[f]);
+                    for (int f = 0; f < NEQ / 2 * 2; f += 2) {
+                        F2 m, q;
+                        linear5_pair(f2(W[0][f], W[0][f + 1]), f2(W[1][f], W[1][f + 1]),
+                                     f2(W[2][f], W[2][f + 1]), f2(W[3][f], W[3][f + 1]), f2(W[4][f], W[4][f + 1]), m, q);
+                        vm[f] = lo(m);
+                        vm[f + 1] = hi(m);
+                        vp[f] = lo(q);
+                        vp[f + 1] = hi(q);
+                    }
+#pragma unroll
+                    for (int f = NEQ / 2 * 2; f < NEQ; ++f) linear5(W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], vm[f], vp[f]);
                     use_weno = !(face_ok<NDIM>(er, vm) && face_ok<NDIM>(er, vp));
                 }
                 if (j >= s0 && j < s1) {   // count each cell once (not the segment halos)
@@ -805,8 +839,37 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
 #pragma unroll
                     for (int f = 0; f < NEQ; ++f) weno5_tab<R>(T, W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], eps, vm[f], vp[f]);
                 } else if (GATED || a.order == 5) {
+                    // two fields at a time as packed pairs, an odd last one by itself
+                    constexpr int PAIRED = PACK ? NEQ / 2 * 2 : 0;
+                    const F2 eps2 = f2(float(eps));
 #pragma unroll
-                    for (int f = 0; f < NEQ; ++f) {
+                    for (int f = 0; f < PAIRED; f += 2) {
+                        F2 m, q;
+                        if constexpr (DCARRY) {
+                            const F2 d3 = f2(Dd3[f], Dd3[f + 1]);
+                            const F2 d4 = sub(f2(W[4][f], W[4][f + 1]), f2(W[3][f], W[3][f + 1]));
+                            const F2 D2 = sub(d4, d3), C2 = mul(mul(f2(c13f), D2), D2);
+                            weno5_dc_pair(f2(W[2][f], W[2][f + 1]), f2(Dd1[f], Dd1[f + 1]), f2(Dd2[f], Dd2[f + 1]), d3,
+                                          d4, f2(Cc0[f], Cc0[f + 1]), f2(Cc1[f], Cc1[f + 1]), C2, eps2, m, q);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                Dd1[f + h] = Dd2[f + h];
+                                Dd2[f + h] = Dd3[f + h];
+                                Dd3[f + h] = h ? hi(d4) : lo(d4);
+                                Cc0[f + h] = Cc1[f + h];
+                                Cc1[f + h] = h ? hi(C2) : lo(C2);
+                            }
+                        } else {
+                            weno5_pair(f2(W[0][f], W[0][f + 1]), f2(W[1][f], W[1][f + 1]), f2(W[2][f], W[2][f + 1]),
+                                       f2(W[3][f], W[3][f + 1]), f2(W[4][f], W[4][f + 1]), eps2, m, q);
+                        }
+                        vm[f] = lo(m);
+                        vm[f + 1] = hi(m);
+                        vp[f] = lo(q);
+                        vp[f + 1] = hi(q);
+                    }
+#pragma unroll
+                    for (int f = PAIRED; f < NEQ; ++f) {
                         if constexpr (DCARRY) {
                             const float d4 = float(W[4][f] - W[3][f]);
                             const float D2 = d4 - Dd3[f];
@@ -825,8 +888,20 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
                         }
                     }
                 } else {   // WENO3 (uniform over the launch): cells i-1 .. i+1 of the window
+                    constexpr int PAIRED = PACK ? NEQ / 2 * 2 : 0;
+                    const F2 eps2 = f2(float(eps));
 #pragma unroll
-                    for (int f = 0; f < NEQ; ++f) {
+                    for (int f = 0; f < PAIRED; f += 2) {
+                        F2 m, q;
+                        weno3_pair(f2(W[1][f], W[1][f + 1]), f2(W[2][f], W[2][f + 1]), f2(W[3][f], W[3][f + 1]), eps2,
+                                   m, q);
+                        vm[f] = lo(m);
+                        vm[f + 1] = hi(m);
+                        vp[f] = lo(q);
+                        vp[f + 1] = hi(q);
+                    }
+#pragma unroll
+                    for (int f = PAIRED; f < NEQ; ++f) {
                         weno3(W[1][f], W[2][f], W[3][f], eps, vm[f], vp[f]);
                     }
                 }

@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kTileThreads, MFC_TILE_BLOCKS) tile_kernel(con
                 double m, q5;
                 if (nu) {
                     const double* T5 = static_cast<const double*>(a.tab) + (long long)(j0 + r) * kTabDoubles;
-                    weno5_tab<double>(T5, v0, v1, v2, v3, v4, a.eps, m, q5);
+                    exact::weno5_tab(T5, v0, v1, v2, v3, v4, a.eps, m, q5);
                 } else if (w5) {
                     const double t2 = exact::curv(v2, v3, v4);
                     exact::weno5_tc(a.eps, v0, v1, v2, v3, v4, t0, t1, t2, p0, p1, m, q5);
