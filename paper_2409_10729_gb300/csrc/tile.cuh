@@ -25,6 +25,7 @@
 // 1024x512 column 6.72 -> 3.36 ms a step; 32^3 RHS 3.9 -> 0.18 ms; 1000-cell
 // tube 2.67 -> 0.041 ms a step.  (256^3 0.411 now, physics_exact.cuh.)
 #pragma once
+#include <algorithm>
 #include <atomic>
 
 #include "sweep.cuh"
@@ -276,33 +277,77 @@ __global__ void __launch_bounds__(kTileThreads, MFC_TILE_BLOCKS) tile_kernel(con
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&a.ctrl->status, 1u);
 }
 
-// Tile of a launch.  P = 4 pencils by the longest J that leaves room for
-// MFC_TILE_BLOCKS tiles in an SM's shared memory (64 cells of 7 fields; the
-// pencil is cut evenly), R = 4.  Where that gives fewer than three tiles per
-// resident block, J is halved down to 16 cells (8 on a single pencil), so that
-// small grids use the whole device, and the runs are shortened, which trades
-// the shared terms for a shorter serial chain.  Measured, FP64: 256^3 P 4, J
-// 64, R 4 0.464 ns per cell, equation and RHS (8, 32, 4: 0.494; 2, 128, 4:
-// 0.470; 4, 64, 8: 0.481; 16, 16, 4: 0.531); 32^3 0.51-0.53 ms a step for 4,
-// 16..32, 1..2 (8, 32, 4: 0.64; 16, 8, 1: 0.60); 1000 cells in 1-D 0.041 ms a
+// Tile of a launch.  Large grids: the split with the least FP64 work per cell, by
+// counting.  A pass over w warps' worth of items costs its warps, and, because a
+// block's four warps meet at a barrier after it, its rounds of four; the FP64
+// instructions of one item are about 8 + 31 R for a run of R reconstructions, 114
+// for a flux, 20 for a conversion and 25 for a cell's end.  P = 4 or 8, pencils
+// cut evenly into up to four pieces more than shared memory asks for, R = 3..9;
+// the estimate is the larger of the rounds and 1.1 times the warps (the FP64 pipe
+// is busy 0.8 of the time at best).  Measured against P = 4, J <= 64, R = 4
+// everywhere: 256^3 144.6 -> 140.0 ms a step, 203^3 80.1 -> 74.9, 160^3 39.3 ->
+// 37.0, 131^3 25.3 -> 24.2, 96^3 10.8 -> 10.5, 1024x512 2.86 -> 2.70 (fixed splits
+// ranged from 140 to 179 ms at 256^3).
+// Grids with fewer than three tiles per resident block at P = 4: J is halved
+// from 64 down to 16 cells (8 on a single pencil), so that small grids use the
+// whole device, and the runs are shortened, which trades the terms that cells
+// share for a shorter serial chain: 32^3 0.454 ms a step with P 4, J 16, R 2 (4,
+// 32, 2: 0.525; 8, 16, 3: 0.545; 2, 16, 2: 0.479); 1000 cells in 1-D 0.041 ms a
 // step for J 8 or 16 (32: 0.052).
 inline TileShape pick_tile(int dir, const int* n, long long ncell, int neq, long long slots) {
     TileShape t;
     const int ns = n[dir];
     t.npen = ncell / ns;
+    auto most_cells = [&](int lp) {   // J that shared memory allows
+        const int ps = lp ? (1 << lp) + 1 : 1;
+        return ((int)(kTileSmem / MFC_TILE_BLOCKS - 1024) / 8 / (neq * ps) - 10) / 3;
+    };
+    auto across = [&](int lp) { return (int)((t.npen + (1LL << lp) - 1) >> lp); };
     t.lp = t.npen >= 4 ? 2 : (t.npen >= 2 ? 1 : 0);
-    t.ntp = (int)((t.npen + (1LL << t.lp) - 1) >> t.lp);
-    const int ps = t.lp ? (1 << t.lp) + 1 : 1;
-    const int room = (int)(kTileSmem / MFC_TILE_BLOCKS - 1024) / 8;
-    int most = (room / (neq * ps) - 10) / 3;
-    if (most > 64) most = 64;
+    t.ntp = across(t.lp);
+    int most = std::min(most_cells(t.lp), 64);
     const int least = t.npen == 1 ? 8 : 16;
     auto tiles = [&](int J) { return (long long)t.ntp * ((ns + J - 1) / J); };
-    while (most / 2 >= least && tiles(most) < 3 * slots) most /= 2;
-    const int nt = (ns + most - 1) / most;
-    t.J = (ns + nt - 1) / nt;
-    const long long nb = tiles(t.J);
-    t.R = nb >= 3 * slots ? 4 : (2 * nb >= slots ? 2 : 1);
+    if (tiles(most) < 3 * slots || t.lp < 2) {
+        while (most / 2 >= least && tiles(most) < 3 * slots) most /= 2;
+        const int nt = (ns + most - 1) / most;
+        t.J = (ns + nt - 1) / nt;
+        const long long nb = tiles(t.J);
+        t.R = nb >= 3 * slots ? 4 : (2 * nb >= slots ? 2 : 1);
+        return t;
+    }
+    double best = 0.0;
+    int blp = 2, bJ = 0, bR = 4;
+    for (int lp = 2; lp <= 3; ++lp) {
+        const int P = 1 << lp, nt0 = (ns + most_cells(lp) - 1) / most_cells(lp);
+        int last = 0;
+        for (int nt = nt0; nt < nt0 + 5; ++nt) {
+            const int J = (ns + nt - 1) / nt;
+            if (J < 8 || J == last) break;
+            last = J;
+            for (int R = 3; R <= 9; ++R) {
+                const int w[4] = {(neq * ((J + 2 + R - 1) / R) * P + 31) / 32, ((J + 1) * P + 31) / 32,
+                                  ((J + 6) * P + 31) / 32, (J * P + 31) / 32};
+                const int c[4] = {8 + 31 * R, 114, 20, 25};
+                int pipe = 0, rounds = 0;
+                for (int k = 0; k < 4; ++k) {
+                    pipe += w[k] * c[k];
+                    rounds += (w[k] + 3) / 4 * 4 * c[k];
+                }
+                const double cost = std::max(1.1 * pipe, (double)rounds) / P * ((ns + J - 1) / J);
+                if (bJ == 0 || cost < best) {
+                    best = cost;
+                    blp = lp;
+                    bJ = J;
+                    bR = R;
+                }
+            }
+        }
+    }
+    t.lp = blp;
+    t.ntp = across(blp);
+    t.J = bJ;
+    t.R = bR;
     return t;
 }
 
