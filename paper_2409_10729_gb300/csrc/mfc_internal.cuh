@@ -225,10 +225,12 @@ __host__ __device__ constexpr bool sweep_balanced(int form, int nf) {
 #ifndef MFC_MIN_BLOCKS_MIXED_X
 #define MFC_MIN_BLOCKS_MIXED_X 2
 #endif
-// 2-D: six fields fit 168 registers (640x320 0.103 -> 0.091 ms a step; in 3-D
-// three blocks cost 512^3 3.41 -> 3.78 ms)
-#ifndef MFC_MIN_BLOCKS_MIXED_X2
-#define MFC_MIN_BLOCKS_MIXED_X2 3
+// x sweeps that fit 168 registers: the 2-D ones with six fields (640x320 0.103 ->
+// 0.091 ms a step) and those on non-uniform grids, which carry no differences
+// (192^3 0.344 -> 0.309 ms); the 3-D one on uniform grids does not (512^3 3.41 ->
+// 3.78 ms)
+#ifndef MFC_MIN_BLOCKS_MIXED_X3
+#define MFC_MIN_BLOCKS_MIXED_X3 3
 #endif
 #ifndef MFC_MIN_BLOCKS_MIXED_RK
 #define MFC_MIN_BLOCKS_MIXED_RK 3

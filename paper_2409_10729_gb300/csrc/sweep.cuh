@@ -492,11 +492,11 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
 // Minimum resident blocks for the register allocator, in blocks of the
 // sweep's own size (x sweeps run one-warp blocks, each with its own output
 // tile in static shared memory).
-template <int FORM, int MODE, int DIR, int NF = 2, int NDIM = 3>
+template <int FORM, int MODE, int DIR, int NF = 2, int NDIM = 3, bool NU = false>
 constexpr int sweep_min_blocks() {
     if (NF > 2) return 1;   // more fields per cell: no register cap (the two-fluid caps spill)
     constexpr int per128 = FORM == FORM_MIXED   ? (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_MIXED_RK
-                                                   : DIR == 0         ? (NDIM == 2 ? MFC_MIN_BLOCKS_MIXED_X2 : MFC_MIN_BLOCKS_MIXED_X)
+                                                   : DIR == 0         ? (NU || NDIM == 2 ? MFC_MIN_BLOCKS_MIXED_X3 : MFC_MIN_BLOCKS_MIXED_X)
                                                                       : MFC_MIN_BLOCKS_MIXED)
                                                 : (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_GATED_RK
                                                    : DIR == 0       ? MFC_MIN_BLOCKS_GATED_X
@@ -507,7 +507,7 @@ constexpr int sweep_min_blocks() {
 // NU: some direction of the grid is non-uniform (tables, per-cell widths);
 // the uniform-grid kernels carry none of that code.
 template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF>
-__global__ void __launch_bounds__(sweep_threads(DIR), sweep_min_blocks<FORM, MODE, DIR, NF, NDIM>())
+__global__ void __launch_bounds__(sweep_threads(DIR), sweep_min_blocks<FORM, MODE, DIR, NF, NDIM, NU>())
 sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
     using R = FormReal<FORM>;
     constexpr bool GATED = FORM == FORM_GATED;
@@ -736,7 +736,9 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
         // mixed form, x sweep: the first differences d1..d3 and curvature parts C0, C1
         // of the window's centre cell, carried along the pencil (weno5_dc); the y and
         // z sweeps, register-capped for occupancy, lose more to spills than it saves
-        // reconstruct two fields at a time (packed FP32 pairs, physics.cuh)
+        // reconstruct two fields at a time (packed FP32 pairs, physics.cuh); from a
+        // table only along x, whose kernel has the registers (elsewhere they spill)
+        constexpr bool TABP = DIR == 0;
         constexpr bool PACK = !NU;
         constexpr bool DCARRY = FORM == FORM_MIXED && !NU && DIR == 0 && MFC_DIFF_CARRY;
         float Dd1[DCARRY ? NEQ : 1], Dd2[DCARRY ? NEQ : 1], Dd3[DCARRY ? NEQ : 1];
@@ -836,8 +838,26 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
             if (use_weno) {
                 if (NU && a.tab) {   // non-uniform direction: this cell's table (uniform over the warp)
                     const R* T = static_cast<const R*>(a.tab) + (long long)(j + 1) * kTabDoubles;
+                    if constexpr (TABP) {
 #pragma unroll
-                    for (int f = 0; f < NEQ; ++f) weno5_tab<R>(T, W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], eps, vm[f], vp[f]);
+                    for (int f = 0; f < NEQ; f += 2) {   // an odd last field is paired with itself
+                        const int g = f + 1 < NEQ ? f + 1 : f;
+                        const R va[5] = {W[0][f], W[1][f], W[2][f], W[3][f], W[4][f]};
+                        const R vb[5] = {W[0][g], W[1][g], W[2][g], W[3][g], W[4][g]};
+                        F2 m, q;
+                        weno5_tab_pair(T, va, vb, f2(float(eps)), m, q);
+                        vm[f] = lo(m);
+                        vp[f] = lo(q);
+                        if (g > f) {
+                            vm[g] = hi(m);
+                            vp[g] = hi(q);
+                        }
+                    }
+                    } else {
+#pragma unroll
+                        for (int f = 0; f < NEQ; ++f)
+                            weno5_tab<R>(T, W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], eps, vm[f], vp[f]);
+                    }
                 } else if (GATED || a.order == 5) {
                     // two fields at a time as packed pairs, an odd last one by itself
                     constexpr int PAIRED = PACK ? NEQ / 2 * 2 : 0;
