@@ -656,7 +656,7 @@ extern "C" int mfc_gate_samples(mfc_ctx* ctx, float* X, float* Y, long long capa
 
 extern "C" int mfc_launches_per_step(mfc_ctx* ctx, int* launches) {
     if (!ctx || !launches) return MFC_EINVAL;
-    *launches = 1 + 3 * ctx->ndim;
+    *launches = 1 + 3 * (ctx->ndim + (split_update(ctx->form, ctx->ndim) ? 1 : 0));
     return MFC_OK;
 }
 

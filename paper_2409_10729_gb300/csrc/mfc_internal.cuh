@@ -141,6 +141,10 @@ constexpr int kTmaCells = 4;
 //   FORM_GATED       FORM_MIXED with the MLP gate (linear weights in smooth cells)
 enum Form { FORM_MIXED = 1, FORM_FP64_EXACT = 2, FORM_GATED = 3 };
 
+// The stage update runs as a kernel of its own after the last sweep (sweep.cuh,
+// stage_update_kernel) instead of inside it.
+__host__ __device__ constexpr bool split_update(int form, int ndim) { return form == FORM_GATED && ndim == 3; }
+
 // Number of parameters of the gate network (W1[32][5], b1, W2[32][32], b2, w3, b3).
 constexpr int kGateParams = 1281;
 

@@ -1158,6 +1158,80 @@ cudaError_t launch_kernel(const SweepArgs& a0, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// SSP-RK3 stage update from the finished accumulator (gated form, 3-D): D_k in
+// FP32, q^(k) = q^n + D_k in FP64, pressure and FP32 copy, and on stage 3 the
+// wave speed of the new state -- what a LAST_RK sweep does with each cell.  As
+// a kernel of its own it streams (172 to 256 bytes a cell at full occupancy),
+// and the z sweep runs as MID at the y sweep's three blocks per SM, where with the
+// update's operands beside stencil and network it had two.  Measured, sweep with
+// update -> sweep + update: gated 256^3 1.531 -> 1.211 ms, 96^3 0.170 -> 0.130,
+// 64^3 0.067 -> 0.071.  The mixed form, whose fused sweep has three blocks, does
+// not gain (512^3 6.69 -> 6.81 ms, 160^3 0.274 -> 0.254, 96^3 0.057 -> 0.069): the
+// accumulator's extra 56 bytes a cell and the launch cost what it saves.
+template <int NDIM>
+__global__ void __launch_bounds__(256) stage_update_kernel(const SweepArgs a) {
+    using FL = Fields<NDIM, 2>;
+    constexpr int NEQ = FL::NEQ, IE = FL::IE;
+    const long long nc = a.ncell, stride = (long long)gridDim.x * blockDim.x;
+    const EosR<float, 2> er(a.eos);
+    const float dt32 = float(a.ctrl->dt), kfac = a.stage == 2 ? 0.25f : (2.0f / 3.0f);
+    const float* acc = static_cast<const float*>(a.acc);
+    float* o32 = static_cast<float*>(a.stage == 3 ? a.qout2 : a.qout);
+    double* o64 = static_cast<double*>(a.qout);
+    float smax = 0.f;
+    bool bad = false;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < nc; c += stride) {
+        float L[NEQ], Dp[NEQ], q32[NEQ];
+        double qnew[NEQ];
+#pragma unroll
+        for (int f = 0; f < NEQ; ++f) {
+            L[f] = acc[f * nc + c];
+            qnew[f] = a.qn[f * nc + c];
+        }
+        if (a.stage != 1) {
+#pragma unroll
+            for (int f = 0; f < NEQ; ++f) Dp[f] = a.dinc[f * nc + c];
+        }
+#pragma unroll
+        for (int f = 0; f < NEQ; ++f) {
+            const float Dk = a.stage == 1 ? dt32 * L[f] : kfac * fmaf(dt32, L[f], Dp[f]);
+            if (a.stage != 3) a.dinc[f * nc + c] = Dk;
+            qnew[f] = qnew[f] + f2d_bits(Dk);
+            q32[f] = d2f_bits(qnew[f]);
+            o32[f * nc + c] = q32[f];
+        }
+        const float pnew = mixed_pressure<NDIM, 2>(a.eos, qnew, q32);
+        o32[NEQ * nc + c] = pnew;
+        if (a.stage == 3) {
+            float v[NEQ], wn[NEQ];
+#pragma unroll
+            for (int f = 0; f < NEQ; ++f) {
+                o64[f * nc + c] = qnew[f];
+                v[f] = q32[f];
+            }
+            v[IE] = pnew;
+            to_prim<NDIM, 2>(er, v, wn);
+            const float s = cell_wavespeed<NDIM, float, 2>(er, wn, a.inv_dx32, bad);
+            smax = s > smax ? s : smax;
+        }
+    }
+    if (a.stage == 3) {
+        const float m = warp_max(smax);
+        if ((threadIdx.x & 31) == 0 && m > 0.f)
+            atomicMax(&a.ctrl->S_bits, (unsigned long long)__double_as_longlong(double(m)));
+        if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(&a.ctrl->status, 1u);
+    }
+}
+
+template <int NDIM>
+cudaError_t launch_stage_update(const SweepArgs& a, cudaStream_t s) {
+    if (a.dry) return cudaSuccess;
+    long long blocks = (a.ncell + 255) / 256;
+    if (blocks > 152LL * 64) blocks = 152LL * 64;
+    stage_update_kernel<NDIM><<<(unsigned)blocks, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 // the FP64 form's sweep (tile.cuh)
 template <int NDIM, int DIR, int MODE, bool NU, int NF>
 cudaError_t launch_tile(const SweepArgs& a, cudaStream_t s);
@@ -1189,7 +1263,12 @@ cudaError_t launch_sweep_t(int dir, int mode, const SweepArgs& a, cudaStream_t s
     } else if (dir == 1 && mode == SW_MID && NDIM == 3) {
         if constexpr (NDIM == 3) return launch_one<NDIM, 1, SW_MID, FORM, NF>(a, s);
     } else if (dir == LAST && mode == SW_LAST_RK) {
-        return launch_one<NDIM, LAST, SW_LAST_RK, FORM, NF>(a, s);
+        if constexpr (split_update(FORM, NDIM)) {
+            const cudaError_t e = launch_one<NDIM, LAST, SW_MID, FORM, NF>(a, s);
+            return e != cudaSuccess ? e : launch_stage_update<NDIM>(a, s);
+        } else {
+            return launch_one<NDIM, LAST, SW_LAST_RK, FORM, NF>(a, s);
+        }
     } else if (dir == LAST && mode == SW_LAST_RHS) {
         return launch_one<NDIM, LAST, SW_LAST_RHS, FORM, NF>(a, s);
     }
