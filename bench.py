@@ -4,8 +4,8 @@
 Metric: grind time, ns per (cell x equation x RHS evaluation), lower is better,
 and the fraction of the HBM roofline it reaches, for the FP64 form (reference
 operation order, bit-identical to the oracle; the headline value), the
-reorganised FP64 form, the mixed-precision form (512^3) and the MLP-gated
-form (256^3, trained weights from paper_2409_10729_gb300/gate_weights.npy),
+FP64-fast selection (the same kernels), the mixed-precision form (512^3) and
+the MLP-gated form (256^3, trained weights from paper_2409_10729_gb300/gate_weights.npy),
 plus the third-order reconstruction option (WENO3-JS) and a tanh-refined
 (non-uniform) grid in the FP64 (256^3) and mixed (512^3) forms, and a
 three-fluid droplet case (256^3, 9 equations) in both.
@@ -171,7 +171,7 @@ def read_traffic(kernel: str):
     import hashlib
     path = os.path.join(ROOT, "profiles", "traffic.txt")
     src = b""
-    for f in ("sweep.cuh", "physics.cuh", "physics_exact.cuh", "mfc_internal.cuh"):
+    for f in ("sweep.cuh", "tile.cuh", "physics.cuh", "physics_exact.cuh", "mfc_internal.cuh"):
         with open(os.path.join(ROOT, "paper_2409_10729_gb300", "csrc", f), "rb") as fh:
             src += fh.read()
     sha = hashlib.sha256(src).hexdigest()[:16]
@@ -275,16 +275,14 @@ def time_form(form, p, w, steps, warmup, device_index, rank, world, kernel_steps
 def roofline_for(form, res, peak_alu, alu_src, hbm_peak, hbm_src):
     """Roofline object for the dominant kernel of one form.
 
-    FP64 forms: the sweeps are bound by the FP64 pipe.  The reference-order
-    form is built without FMA contraction, so every algorithmic +, -, *, /,
-    sqrt issues at least one FP64 instruction, and its ceiling is the FP64
-    instruction rate: the FMA-chain probe's FMA instructions per second (its
-    TFLOP/s over 2).  achieved = algorithmic operations per second; the gap
-    to ncu's FP64 pipe-busy fraction is what a correctly rounded division or
-    square root costs beyond its one algorithmic operation.  The reorganised
-    FP64 form and the FP32 forms are built with FMA contraction: their
-    ceiling is the probe's TFLOP/s at 2 flops per FMA (FP64 and FP32 probe
-    respectively)."""
+    FP64 form: the sweeps are bound by the FP64 pipe, whose rate is the
+    FMA-chain probe's FMA instructions per second (its TFLOP/s over 2).
+    achieved = algorithmic +, -, *, /, sqrt per second.  The quotients, square
+    roots and WENO's products are formed on the integer pipes, about half of
+    the algorithmic operations, so the fraction of that rate can pass 1; how
+    busy the pipe itself is, ncu says (pipe_busy_ncu).  The FP64-fast entry runs
+    the same kernels and is held, as before, against 2 flops per FMA; so are
+    the FP32 forms, against the FP32 probe."""
     kt = res["kernels"]
     base = form.replace("_weno3", "").replace("_stretched", "").replace("_3fluid", "")
     name = max((k for k in kt if kt[k][1] > 0), key=lambda k: kt[k][0])
@@ -302,7 +300,8 @@ def roofline_for(form, res, peak_alu, alu_src, hbm_peak, hbm_src):
     if base == "fp64":   # the reference-order form (no FMA contraction)
         peak, unit = peak_alu / 2.0, "Top/s"
         src = (f"{alu_src}: {peak_alu:.3f} TFLOP/s = {peak_alu / 2:.3f} T FP64 FMA instructions/s; one algorithmic "
-               "operation (+, -, *, /, sqrt, min/max) per FP64 instruction slot")
+               "operation (+, -, *, /, sqrt, min/max) per FP64 instruction slot; those formed on the integer "
+               "pipes take none, so the fraction can pass 1")
     else:
         peak, unit = peak_alu, "TFLOP/s"
         src = f"{alu_src} ({'FP64' if base == 'fp64_fast' else 'FP32'}, 2 flops per FMA)"

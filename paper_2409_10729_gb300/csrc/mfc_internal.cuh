@@ -87,7 +87,7 @@ struct SweepArgs {
     float* dinc;          // FP32 forms: the RK increment D_k of the stage (neq fields), read and rewritten
     int n[3];
     long long ncell;
-    double inv_dx[3];     // n/(hi - lo) per direction (reformulated forms)
+    double inv_dx[3];     // n/(hi - lo) per direction
     double dx[3];         // (hi - lo)/n per direction
     double rdx[3];        // RN(1/dx) per direction (reference-order form)
     float inv_dx32[3];    // inv_dx rounded to FP32 (FP32 forms)

@@ -1,17 +1,16 @@
-// physics.cuh -- device-side arithmetic of the five-equation RHS.
+// physics.cuh -- device-side arithmetic of the five-equation RHS, FP32 forms, and
+// what both precisions share (EOS constants, field layout, compares).
 //
-// Stiffened-gas mixture EOS (arXiv 2409.10729, Sec. II-A), WENO5-JS face
-// reconstruction and the HLLC flux (Sec. II-B, last paragraph), written for
-// the GB300 FP64 and FP32 pipes.  The formulas are the same as the serial
-// oracle's, reorganised to spend fewer divisions, which are the expensive
-// operations on this part:
-//   * WENO weights in product form: omega_k ~ d_k * prod_{j != k} (eps+beta_j)^2,
-//     so each face value costs one division instead of six (FP64), or
-//     min-normalised reciprocals that cannot overflow (FP32);
+// Stiffened-gas mixture EOS (arXiv 2409.10729, Sec. II-A), WENO-JS face
+// reconstruction and the HLLC flux (Sec. II-B, last paragraph).  The formulas
+// are the same as the serial oracle's, reorganised to spend fewer divisions:
+//   * WENO weights relative to the smoothest stencil, by reciprocals that cannot
+//     overflow, and one reciprocal per face;
 //   * candidate stencils multiplied by 1/6 instead of divided by 6;
 //   * the HLLC star energy uses one reciprocal 1/(S_K - S*) for both chi_K
 //     and the p_K/(S_K - u_K) term.
-// Results agree with the oracle to rounding, not bit for bit.
+// Results agree with the oracle to FP32 rounding.  The FP64 form's arithmetic is
+// in physics_exact.cuh.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -162,9 +161,8 @@ __device__ __forceinline__ void mixture(const EosR<R, NF>& e, const R* a, R& G, 
 //   left:  (5 d2 - 2 d1)/6, (d2 + 2 d3)/6, (4 d3 - d4)/6
 //   right: (d1 - 4 d2)/6, -(2 d2 + d3)/6, (2 d4 - 5 d3)/6
 // (the same polynomials as the textbook forms), so uniform data reconstructs
-// exactly.  FP64: product-form weights and one reciprocal for both faces.
-// FP32: weights relative to the smoothest stencil, the linear weights and
-// the 1/6 folded into the corrections, one fast reciprocal per face.
+// exactly.  Weights relative to the smoothest stencil, the linear weights and the
+// 1/6 folded into the corrections, one fast reciprocal per face.
 // FP32 WENO5 from the smoothness indicators: weights relative to the smoothest
 // stencil, the linear weights and the 1/6 of the candidates folded into the
 // corrections, one reciprocal per face.
@@ -329,15 +327,9 @@ __device__ __forceinline__ void weno3(R v1, R v2, R v3, R eps, R& vm, R& vp) {
     R s0 = eps + d1 * d1, s1 = eps + d2 * d2;
     s0 = s0 * s0;
     s1 = s1 * s1;
-    R m0, m1;
-    if constexpr (sizeof(R) == 8) {
-        m0 = s1;   // product form: weight of stencil k proportional to d_k * s_other
-        m1 = s0;
-    } else {
-        R smin = fminf(s0, s1);
-        m0 = __fdividef(smin, s0);
-        m1 = __fdividef(smin, s1);
-    }
+    R smin = fminf(s0, s1);
+    R m0 = __fdividef(smin, s0);
+    R m1 = __fdividef(smin, s1);
     R am0 = R(1.0 / 3.0) * m0, am1 = R(2.0 / 3.0) * m1;
     R ap0 = R(2.0 / 3.0) * m0, ap1 = R(1.0 / 3.0) * m1;
     R Dm = am0 + am1, Dp = ap0 + ap1;
@@ -400,8 +392,7 @@ __device__ __forceinline__ void weno5_tab_pair(const float* __restrict__ T, cons
 // WENO5-JS on a non-uniform grid from the cell's table T (kTabDoubles values,
 // the same for every lane of a warp): candidates q_k^+- = cp_k.v, cm_k.v,
 // smoothness beta_k = (B_k.v)^2 + 13/3 (C_k.v)^2, linear weights dp, dm;
-// weights scaled as in weno5 (product form in FP64, relative to the smoothest
-// stencil in FP32), one reciprocal for both faces.
+// weights relative to the smoothest stencil, one reciprocal for both faces.
 template <typename R>
 __device__ __forceinline__ void weno5_tab(const R* __restrict__ T, R v0, R v1, R v2, R v3, R v4, R eps, R& vm,
                                           R& vp) {
@@ -423,17 +414,10 @@ __device__ __forceinline__ void weno5_tab(const R* __restrict__ T, R v0, R v1, R
         const R beta = c * c + R(13.0 / 3.0) * (d * d);
         s[k] = (eps + beta) * (eps + beta);
     }
-    R m0, m1, m2;
-    if constexpr (sizeof(R) == 8) {
-        m0 = s[1] * s[2];
-        m1 = s[0] * s[2];
-        m2 = s[0] * s[1];
-    } else {
-        R smin = fminf(s[0], fminf(s[1], s[2]));
-        m0 = __fdividef(smin, s[0]);
-        m1 = __fdividef(smin, s[1]);
-        m2 = __fdividef(smin, s[2]);
-    }
+    R smin = fminf(s[0], fminf(s[1], s[2]));
+    R m0 = __fdividef(smin, s[0]);
+    R m1 = __fdividef(smin, s[1]);
+    R m2 = __fdividef(smin, s[2]);
     const R ap0 = __ldg(T + 36) * m0, ap1 = __ldg(T + 37) * m1, ap2 = __ldg(T + 38) * m2;
     const R am0 = __ldg(T + 39) * m0, am1 = __ldg(T + 40) * m1, am2 = __ldg(T + 41) * m2;
     const R Dp = ap0 + ap1 + ap2, Dm = am0 + am1 + am2;
