@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stddef.h>
+#include <stdint.h>
 #include <stdlib.h>
 #include <string.h>
 
@@ -391,8 +392,12 @@ static cudaError_t set_state_from(mfc_ctx* ctx, const double* src, bool prim, fl
 
 static int set_state_impl(mfc_ctx* ctx, const double* src, int on_device, bool prim) {
     if (!ctx || !src) return MFC_EINVAL;
+    const size_t bytes = (size_t)ctx->ncell * ctx->neq * sizeof(double);
     if (!on_device) {
-        CK(host_copy(ctx->qn, src, (size_t)ctx->ncell * ctx->neq * sizeof(double), true, ctx->stream));
+        CK(host_copy(ctx->qn, src, bytes, true, ctx->stream));
+        src = ctx->qn;
+    } else if ((uintptr_t)src % sizeof(double) != 0) {   // the kernel reads doubles
+        CK(cudaMemcpyAsync(ctx->qn, src, bytes, cudaMemcpyDeviceToDevice, ctx->stream));
         src = ctx->qn;
     }
     CK(set_state_from(ctx, src, prim, fp32_state(ctx) ? ctx->s0 : NULL));

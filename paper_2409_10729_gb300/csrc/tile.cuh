@@ -318,12 +318,12 @@ inline TileShape pick_tile(int dir, const int* n, long long ncell, int neq, long
     }
     double best = 0.0;
     int blp = 2, bJ = 0, bR = 4;
-    for (int lp = 2; lp <= 3; ++lp) {
+    for (int lp = 2; lp <= 3 && (1LL << lp) <= t.npen; ++lp) {
         const int P = 1 << lp, nt0 = (ns + most_cells(lp) - 1) / most_cells(lp);
         int last = 0;
         for (int nt = nt0; nt < nt0 + 5; ++nt) {
             const int J = (ns + nt - 1) / nt;
-            if (J < 8 || J == last) break;
+            if (nt > nt0 && (J < 8 || J == last)) break;
             last = J;
             for (int R = 3; R <= 9; ++R) {
                 const int w[4] = {(neq * ((J + 2 + R - 1) / R) * P + 31) / 32, ((J + 1) * P + 31) / 32,
@@ -334,7 +334,7 @@ inline TileShape pick_tile(int dir, const int* n, long long ncell, int neq, long
                     pipe += w[k] * c[k];
                     rounds += (w[k] + 3) / 4 * 4 * c[k];
                 }
-                const double cost = std::max(1.1 * pipe, (double)rounds) / P * ((ns + J - 1) / J);
+                const double cost = std::max(1.1 * pipe, (double)rounds) * across(lp) * ((ns + J - 1) / J);
                 if (bJ == 0 || cost < best) {
                     best = cost;
                     blp = lp;

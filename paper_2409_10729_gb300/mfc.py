@@ -369,15 +369,15 @@ def _stream() -> int:
 
 
 def mlp_loss_grad(X, Y, theta, grad, loss, pos_weight: float = 1.0):
-    st = (_lib or lib()).mfc_mlp_loss_grad(X.data_ptr(), Y.data_ptr(), Y.numel(), theta.data_ptr(), pos_weight,
+    st = (_lib or lib()).mfc_mlp_loss_grad(X.data_ptr(), Y.data_ptr(), Y.numel(), theta.data_ptr(), float(pos_weight),
                                            grad.data_ptr(), loss.data_ptr(), _stream())
     if st != MFC_OK:
         raise MfcError(st, "mfc_mlp_loss_grad")
 
 
 def mlp_adam(theta, grad, m, v, t: int, lr=1e-3, beta1=0.9, beta2=0.999, eps=1e-8):
-    st = (_lib or lib()).mfc_mlp_adam(theta.data_ptr(), grad.data_ptr(), m.data_ptr(), v.data_ptr(), int(t), lr, beta1,
-                                      beta2, eps, _stream())
+    st = (_lib or lib()).mfc_mlp_adam(theta.data_ptr(), grad.data_ptr(), m.data_ptr(), v.data_ptr(), int(t), float(lr),
+                                      float(beta1), float(beta2), float(eps), _stream())
     if st != MFC_OK:
         raise MfcError(st, "mfc_mlp_adam")
 
