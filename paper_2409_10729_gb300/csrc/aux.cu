@@ -317,6 +317,14 @@ __global__ void exact_ops_check_kernel(long long n, unsigned long long seed, uns
         else if (pick == 2u) w = bits ^ 0x8000000000000000ULL;
         else if ((w & 7u) == 0u) w &= 0x8000000000000000ULL;   // +-0 now and then
         const double y = __longlong_as_double((long long)w);
+        // the general forms on any operands
+        bool norm = true;
+        const double pw = mul_s(x, y, norm), ph = __dmul_rn(x, y);
+        bad += norm && __double_as_longlong(pw) != __double_as_longlong(ph);
+        const double qw = quot(x, y), qh = __ddiv_rn(x, y);
+        bad += __double_as_longlong(qw) != __double_as_longlong(qh) && !(qw != qw && qh != qh);
+        const double rw = sqrt_p(x), rh = __dsqrt_rn(x);
+        bad += __double_as_longlong(rw) != __double_as_longlong(rh) && !(rw != rw && rh != rh);
         bad += (gt0(x) != (x > 0.0)) + (ge0(x) != (0.0 <= x)) + (less(x, y) != (x < y)) + (less(y, x) != (y < x));
         // quotients from significands: operands moved into the range of
         // mid_range, some with a significand next to a power of two, and the

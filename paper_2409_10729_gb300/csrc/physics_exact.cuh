@@ -154,40 +154,47 @@ __device__ __forceinline__ bool in_range(double x) {
     return (((unsigned)__double2hiint(x) & 0x7fffffffu) - ((1023u - R) << 20)) < ((2u * R) << 20);
 }
 
-// RN(x^2) for x zero or within 2^-300 .. 2^300 (else ok is cleared)
+// Normal: neither zero, subnormal, infinite nor NaN; h: the number's high word
+__device__ __forceinline__ bool normal_hi(unsigned h) { return (h & 0x7ff00000u) - 0x00100000u < 0x7fe00000u; }
+
+// RN(x^2) for |x| within 2^-300 .. 2^300; smaller x give 0, larger ones and NaN
+// clear ok.  (The squares of differences below 2^-300 are parts of smoothness
+// indicators, added to an eps whose own square is a normal number, at least
+// 2^-511: they are below half a unit in the last place of any such sum.)
 __device__ __forceinline__ double sq_i(double x, bool& ok) {
-    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
-    const bool zero = ((h << 1) | l) == 0u;
-    ok = ok && (zero || in_range<300>(x));
+    const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu, l = (unsigned)__double2loint(x);
+    ok = ok && h < (1323u << 20);
     const unsigned m = (h & 0x000fffffu) | 0x00100000u;
     const unsigned long long t0 = wide(l, l), t1 = wide(l, m << 1) + hi32(t0), t2 = wide(m, m) + hi32(t1);
     const double r = round_product(hi32(t2), lo32(t2), lo32(t1), lo32(t0), 2u * (h & 0x7ff00000u) - (1024u << 20));
-    return zero ? 0.0 : r;
+    return h < (723u << 20) ? 0.0 : r;
 }
 
-// RN(a b) for a positive within 2^-300 .. 2^300 and b zero or of a size within
-// that range (else ok is cleared; a is the caller's to check)
+// RN(a b) for a positive and normal and b zero, or b and the product normal (else
+// ok is cleared; a is the caller's to check)
 __device__ __forceinline__ double mul_i(double a, double b, bool& ok) {
     const unsigned ha = (unsigned)__double2hiint(a), la = (unsigned)__double2loint(a);
     const unsigned hb = (unsigned)__double2hiint(b), lb = (unsigned)__double2loint(b);
     const bool zero = ((hb << 1) | lb) == 0u;
-    ok = ok && (zero || in_range<300>(b));
+    const unsigned e20 = (ha & 0x7ff00000u) + (hb & 0x7ff00000u) - (1024u << 20);
+    ok = ok && (zero || (normal_hi(hb) && e20 < (2044u << 20)));
     const unsigned ma = (ha & 0x000fffffu) | 0x00100000u, mb = (hb & 0x000fffffu) | 0x00100000u;
     const unsigned long long t0 = wide(la, lb), t1 = wide(la, mb) + hi32(t0), t2 = wide(ma, lb) + lo32(t1);
     const unsigned long long t3 = wide(ma, mb) + (hi32(t1) + hi32(t2));
-    const double r = round_product(hi32(t3), lo32(t3), lo32(t2), lo32(t0),
-                                   (ha & 0x7ff00000u) + (hb & 0x7ff00000u) - (1024u << 20));
+    const double r = round_product(hi32(t3), lo32(t3), lo32(t2), lo32(t0), e20);
     const unsigned sign = hb & 0x80000000u;
     return __hiloint2double((int)((zero ? 0u : (unsigned)__double2hiint(r)) | sign),
                             (int)(zero ? 0u : (unsigned)__double2loint(r)));
 }
 
-// RN(a b) for a and b each zero or within 2^-300 .. 2^300 in size (else ok is cleared)
+// RN(a b) for a and b each zero, or both and the product normal (else ok is cleared)
 __device__ __forceinline__ double mul_s(double a, double b, bool& ok) {
     const unsigned ha = (unsigned)__double2hiint(a), la = (unsigned)__double2loint(a);
     const bool zero = ((ha << 1) | la) == 0u;
-    ok = ok && (zero || in_range<300>(a));
-    const double r = mul_i(a, b, ok);   // the sign of b
+    bool in = normal_hi(ha);
+    const double r = mul_i(a, b, in);   // the sign of b
+    const unsigned hb = (unsigned)__double2hiint(b);
+    ok = ok && (in || (zero && (hb & 0x7ff00000u) != 0x7ff00000u));
     const unsigned h = (unsigned)__double2hiint(r);
     return __hiloint2double((int)((zero ? h & 0x80000000u : h) ^ (ha & 0x80000000u)),
                             zero ? 0 : __double2loint(r));
@@ -255,18 +262,21 @@ __device__ __forceinline__ double sqrt_p(double a) {
 }
 
 // RN(a/b) for any a and b, y = rcp_i(b): signs and a zero numerator are dealt
-// with here, operands outside the middle of the range take the FP64 division.
+// with here, operands or quotients that are not normal take the FP64 division.
+// (Disturbances run ahead of a front by many orders of magnitude a cell, so tiny
+// normal numbers are common: while anything below 2^-300 took the FP64 path,
+// here and in the squares and products, 256^3 droplets took 154 ms a step after
+// twelve steps, 139 now, and 142 -> 134 at the start.)
 __device__ __forceinline__ double quot(double a, double b, const RcpI& y) {
     const unsigned ha = (unsigned)__double2hiint(a), la = (unsigned)__double2loint(a);
     const unsigned hb = (unsigned)__double2hiint(b);
     const bool zero = ((ha << 1) | la) == 0u;
-    const bool in = ((ha & 0x7fffffffu) - (723u << 20)) < (600u << 20);
-    const bool bin = ((hb & 0x7fffffffu) - (723u << 20)) < (600u << 20);
+    const bool in = normal_hi(ha) && (ha & 0x7ff00000u) - y.e20 + (1021u << 20) < (2044u << 20);
     const double q = quot_i(a, y);
     const unsigned sign = (ha ^ hb) & 0x80000000u;
     double r = __hiloint2double((int)((zero ? 0u : (unsigned)__double2hiint(q)) | sign),
                                 (int)(zero ? 0u : (unsigned)__double2loint(q)));
-    if (__builtin_expect(!(bin && (in || zero)), 0)) r = div_any(a, b);
+    if (__builtin_expect(!(normal_hi(hb) && (in || zero)), 0)) r = div_any(a, b);
     return r;
 }
 __device__ __forceinline__ double quot(double a, double b) { return quot(a, b, rcp_i(b)); }
