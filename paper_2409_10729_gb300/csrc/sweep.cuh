@@ -733,13 +733,15 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
             to_prim<NDIM, NF>(er, v, W[k]);
             bad |= !pos(mix_rho<NF>(W[k]));
         }
+        // reconstruct two fields at a time (packed FP32 pairs, physics.cuh), not in
+        // 1-D, where one dependent chain per warp is all there is (2122 cells 4%
+        // slower); from a table only along x, whose kernel has the registers
+        // (elsewhere they spill)
+        constexpr bool TABP = DIR == 0 && NDIM > 1;
+        constexpr bool PACK = !NU && NDIM > 1;
         // mixed form, x sweep: the first differences d1..d3 and curvature parts C0, C1
         // of the window's centre cell, carried along the pencil (weno5_dc); the y and
         // z sweeps, register-capped for occupancy, lose more to spills than it saves
-        // reconstruct two fields at a time (packed FP32 pairs, physics.cuh); from a
-        // table only along x, whose kernel has the registers (elsewhere they spill)
-        constexpr bool TABP = DIR == 0;
-        constexpr bool PACK = !NU;
         constexpr bool DCARRY = FORM == FORM_MIXED && !NU && DIR == 0 && MFC_DIFF_CARRY;
         float Dd1[DCARRY ? NEQ : 1], Dd2[DCARRY ? NEQ : 1], Dd3[DCARRY ? NEQ : 1];
         float Cc0[DCARRY ? NEQ : 1], Cc1[DCARRY ? NEQ : 1];
@@ -814,7 +816,7 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
                 const bool smooth = (!live_r || zr < 0.f) && (!live_p || zp < 0.f);
                 if (smooth) {
 #pragma unroll
-                    for (int f = 0; f < NEQ / 2 * 2; f += 2) {
+                    for (int f = 0; f < (PACK ? NEQ / 2 * 2 : 0); f += 2) {
                         F2 m, q;
                         linear5_pair(f2(W[0][f], W[0][f + 1]), f2(W[1][f], W[1][f + 1]),
                                      f2(W[2][f], W[2][f + 1]), f2(W[3][f], W[3][f + 1]), f2(W[4][f], W[4][f + 1]), m, q);
@@ -824,7 +826,7 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
                         vp[f + 1] = hi(q);
                     }
 #pragma unroll
-                    for (int f = NEQ / 2 * 2; f < NEQ; ++f) linear5(W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], vm[f], vp[f]);
+                    for (int f = PACK ? NEQ / 2 * 2 : 0; f < NEQ; ++f) linear5(W[0][f], W[1][f], W[2][f], W[3][f], W[4][f], vm[f], vp[f]);
                     use_weno = !(face_ok<NDIM>(er, vm) && face_ok<NDIM>(er, vp));
                 }
                 if (j >= s0 && j < s1) {   // count each cell once (not the segment halos)
