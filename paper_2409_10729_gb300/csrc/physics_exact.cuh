@@ -192,12 +192,12 @@ __device__ __forceinline__ double mul_s(double a, double b, bool& ok) {
     const unsigned ha = (unsigned)__double2hiint(a), la = (unsigned)__double2loint(a);
     const bool zero = ((ha << 1) | la) == 0u;
     bool in = normal_hi(ha);
-    const double r = mul_i(a, b, in);   // the sign of b
+    const double r = mul_i(a, b, in);
     const unsigned hb = (unsigned)__double2hiint(b);
     ok = ok && (in || (zero && (hb & 0x7ff00000u) != 0x7ff00000u));
-    const unsigned h = (unsigned)__double2hiint(r);
-    return __hiloint2double((int)((zero ? h & 0x80000000u : h) ^ (ha & 0x80000000u)),
-                            zero ? 0 : __double2loint(r));
+    // the sign from the operands: with a zero, r's high word means nothing
+    const unsigned h = zero ? 0u : (unsigned)__double2hiint(r) & 0x7fffffffu;
+    return __hiloint2double((int)(h | ((ha ^ hb) & 0x80000000u)), zero ? 0 : __double2loint(r));
 }
 
 // How the EOS functions below form their products: on the FP64 pipe, or on the
