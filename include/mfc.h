@@ -22,7 +22,9 @@
  *     memory pinned by PyTorch, under unified addressing), with its address
  *     and size multiples of 16 bytes, is copied by the GPU's SMs through that
  *     mapping; it must lie within one page-locked allocation.  Other host
- *     memory goes through cudaMemcpyAsync.
+ *     memory goes through cudaMemcpyAsync.  The state setters read an array
+ *     in this device's memory in place; an on_device array anywhere else
+ *     (another GPU's memory, say) they copy first.
  *   - The context owns all device memory it allocates; the caller owns every
  *     pointer it passes in and keeps it valid until the call returns.
  *   - Every call returns an mfc_status.  Nothing aborts, traps or prints.

@@ -16,6 +16,7 @@
 
 #include "mfc.h"
 #include "mfc_internal.cuh"
+#include "state_source.h"
 
 using namespace mfc5;
 
@@ -165,6 +166,42 @@ static EncodeTiledFn encode_tiled() {
             cudaGetLastError();
     }
     return fn;
+}
+
+typedef CUresult (*PointerAttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+
+// What the driver knows of a device address (zeros where the query fails).
+static PointerInfo pointer_info(const void* ptr) {
+    static const PointerAttributesFn fn = [] {
+        void* f = NULL;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) !=
+                cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = NULL;
+        }
+        return (PointerAttributesFn)f;
+    }();
+    PointerInfo o = {};
+    if (!fn) return o;
+    unsigned int type = 0, managed = 0;
+    int device = -1;
+    CUdeviceptr range = 0, map = 0;
+    size_t range_bytes = 0, map_bytes = 0;
+    CUpointer_attribute at[7] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                 CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                 CU_POINTER_ATTRIBUTE_RANGE_SIZE, CU_POINTER_ATTRIBUTE_MAPPING_BASE_ADDR,
+                                 CU_POINTER_ATTRIBUTE_MAPPING_SIZE};
+    void* out[7] = {&type, &managed, &device, &range, &range_bytes, &map, &map_bytes};
+    if (fn(7, at, out, (CUdeviceptr)ptr) != CUDA_SUCCESS) return o;
+    o.device_memory = type == CU_MEMORYTYPE_DEVICE && !managed;
+    o.device = device;
+    o.range = (uintptr_t)range;
+    o.range_bytes = range_bytes;
+    o.map = (uintptr_t)map;
+    o.map_bytes = map_bytes;
+    return o;
 }
 
 // Tensor maps of an FP32 stage buffer [field][z][y][x] as a 4-D tensor
@@ -396,7 +433,7 @@ static int set_state_impl(mfc_ctx* ctx, const double* src, int on_device, bool p
     if (!on_device) {
         CK(host_copy(ctx->qn, src, bytes, true, ctx->stream));
         src = ctx->qn;
-    } else if ((uintptr_t)src % sizeof(double) != 0) {   // the kernel reads doubles
+    } else if (!read_in_place(pointer_info(src), (uintptr_t)src, bytes, ctx->device)) {
         CK(cudaMemcpyAsync(ctx->qn, src, bytes, cudaMemcpyDeviceToDevice, ctx->stream));
         src = ctx->qn;
     }
