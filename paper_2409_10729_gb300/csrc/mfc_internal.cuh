@@ -232,7 +232,7 @@ __host__ __device__ constexpr bool sweep_balanced(int form, int nf) {
 // x sweeps that fit 168 registers: the 2-D ones with six fields (640x320 0.103 ->
 // 0.091 ms a step) and those on non-uniform grids, which carry no differences
 // (192^3 0.344 -> 0.309 ms); the 3-D one on uniform grids does not (512^3 3.41 ->
-// 3.78 ms)
+// 3.78 ms).  Not where the third block saves no wave: take_lean.
 #ifndef MFC_MIN_BLOCKS_MIXED_X3
 #define MFC_MIN_BLOCKS_MIXED_X3 3
 #endif
@@ -250,6 +250,48 @@ __host__ __device__ constexpr bool sweep_balanced(int form, int nf) {
 #ifndef MFC_MIN_BLOCKS_GATED_RK
 #define MFC_MIN_BLOCKS_GATED_RK 2
 #endif
+// Lean kernels of the mixed form: the same sweep with one field per instruction
+// instead of packed pairs (uniform grids), and along x with two blocks per SM where
+// the full kernel has three.  Both give the same bits.  Packing and the third block
+// buy throughput and pay with registers and longer dependent chains, so the lean
+// kernel stays where a launch does not fill the device or the registers run out.
+enum LeanUse { LEAN_NEVER, LEAN_ALWAYS, LEAN_BY_LAUNCH };
+
+// Four fluids along x: packed, 160 (3-D) and 212 bytes (2-D) spill at 255 registers;
+// 160^3 WENO5 246 -> 241 us, WENO3 241 -> 231; 1021x515 WENO3 56.8 -> 46.6.  (2-D WENO5
+// was 1 to 4% better packed: 512x256 42.4, 43.8.)  Three fluids along x in 3-D gain by
+// packing (160^3 184 -> 175), in 2-D only with WENO5.
+__host__ __device__ constexpr LeanUse lean_use(int form, int ndim, int dir, bool nu, int nf) {
+    if (form != FORM_MIXED || ndim == 1) return LEAN_NEVER;
+    if (nu) return dir == 0 ? LEAN_BY_LAUNCH : LEAN_NEVER;
+    if (nf == 2) return LEAN_BY_LAUNCH;
+    if (dir != 0) return LEAN_NEVER;
+    return nf == 4 ? LEAN_ALWAYS : (ndim == 2 ? LEAN_BY_LAUNCH : LEAN_NEVER);
+}
+
+// What a launch would put on the device: its blocks, and the blocks resident at once.
+struct LaunchFill {
+    long long blocks, slots;
+    long long waves() const { return (blocks + slots - 1) / slots; }
+};
+
+// Measured, lean against full:
+//   non-uniform, x sweep: the third block pays when it saves a wave (96^3 70 -> 50 us,
+//     203x149x97 204 -> 184, 256^3 780 -> 702), else it costs (128^3 123 -> 135)
+//   WENO5, uniform: full everywhere
+//   WENO3, three fluids (2-D, x): lean (1021x515 39.2, 41.2 us full)
+//   WENO3, two fluids, 2-D x sweep: as non-uniform (640x320 22.0 -> 16.6 us; 2048x1024
+//     68.2 -> 72.2; 64x48 57.0 -> 59.5 a step)
+//   WENO3, two fluids, elsewhere: full from half a wave on (us a step: 16^3 80.4 -> 81.7,
+//     32^3 86.6 -> 88.6, 48^3 equal, 64^3 178 -> 175, 160^3 1501 -> 1469)
+inline bool take_lean(int ndim, int dir, bool nu, int nf, int order, const LaunchFill& lean, const LaunchFill& full) {
+    if (nu) return lean.waves() <= full.waves();
+    if (order != 3) return false;
+    if (nf > 2) return true;
+    if (dir == 0 && ndim == 2) return lean.waves() <= full.waves();
+    return 2 * full.blocks <= full.slots;
+}
+
 // 1: the sweeps issue the loads of the cell entering the stencil window at the
 // top of each step along the pencil (they complete under that step's
 // arithmetic); 0: at the bottom, just before they are used.

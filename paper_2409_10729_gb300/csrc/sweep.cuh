@@ -492,11 +492,11 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
 // Minimum resident blocks for the register allocator, in blocks of the
 // sweep's own size (x sweeps run one-warp blocks, each with its own output
 // tile in static shared memory).
-template <int FORM, int MODE, int DIR, int NF = 2, int NDIM = 3, bool NU = false>
+template <int FORM, int MODE, int DIR, int NF = 2, int NDIM = 3, bool NU = false, bool LEAN = false>
 constexpr int sweep_min_blocks() {
     if (NF > 2) return 1;   // more fields per cell: no register cap (the two-fluid caps spill)
     constexpr int per128 = FORM == FORM_MIXED   ? (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_MIXED_RK
-                                                   : DIR == 0         ? (NU || NDIM == 2 ? MFC_MIN_BLOCKS_MIXED_X3 : MFC_MIN_BLOCKS_MIXED_X)
+                                                   : DIR == 0         ? ((NU || NDIM == 2) && !LEAN ? MFC_MIN_BLOCKS_MIXED_X3 : MFC_MIN_BLOCKS_MIXED_X)
                                                                       : MFC_MIN_BLOCKS_MIXED)
                                                 : (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_GATED_RK
                                                    : DIR == 0       ? MFC_MIN_BLOCKS_GATED_X
@@ -505,9 +505,10 @@ constexpr int sweep_min_blocks() {
 }
 
 // NU: some direction of the grid is non-uniform (tables, per-cell widths);
-// the uniform-grid kernels carry none of that code.
-template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF>
-__global__ void __launch_bounds__(sweep_threads(DIR), sweep_min_blocks<FORM, MODE, DIR, NF, NDIM, NU>())
+// the uniform-grid kernels carry none of that code.  LEAN: the mixed form's
+// second kernel of a sweep (lean_use, mfc_internal.cuh).
+template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF, bool LEAN>
+__global__ void __launch_bounds__(sweep_threads(DIR), sweep_min_blocks<FORM, MODE, DIR, NF, NDIM, NU, LEAN>())
 sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
     using R = FormReal<FORM>;
     constexpr bool GATED = FORM == FORM_GATED;
@@ -736,9 +737,9 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
         // reconstruct two fields at a time (packed FP32 pairs, physics.cuh), not in
         // 1-D, where one dependent chain per warp is all there is (2122 cells 4%
         // slower); from a table only along x, whose kernel has the registers
-        // (elsewhere they spill)
+        // (elsewhere they spill), and not in lean kernels
         constexpr bool TABP = DIR == 0 && NDIM > 1;
-        constexpr bool PACK = !NU && NDIM > 1;
+        constexpr bool PACK = !NU && NDIM > 1 && !LEAN;
         // mixed form, x sweep: the first differences d1..d3 and curvature parts C0, C1
         // of the window's centre cell, carried along the pencil (weno5_dc); the y and
         // z sweeps, register-capped for occupancy, lose more to spills than it saves
@@ -1092,7 +1093,7 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
 
 // Resident blocks of one sweep kernel on the current device (occupancy x
 // SMs), looked up once per kernel and device (devices may differ in SM count).
-template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF>
+template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF, bool LEAN>
 long long sweep_slots() {
     constexpr int kMaxDev = 64;
     static long long cache[kMaxDev];   // 0: not yet looked up (a benign race: every writer stores the same value)
@@ -1103,7 +1104,7 @@ long long sweep_slots() {
     }
     if (dev >= 0 && dev < kMaxDev && cache[dev] > 0) return cache[dev];
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel<NDIM, DIR, MODE, FORM, NU, NF>,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sweep_kernel<NDIM, DIR, MODE, FORM, NU, NF, LEAN>,
                                                       sweep_threads(DIR), 0) != cudaSuccess) {
         cudaGetLastError();
         per_sm = 1;
@@ -1128,14 +1129,12 @@ inline int pick_seg(int dir, const int* n, int threads, long long slots) {
     return seg;
 }
 
+// A launch's mapping of cells to warps (a.nwarps, a.seg) and its blocks.
 template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF>
-cudaError_t launch_kernel(const SweepArgs& a0, cudaStream_t s) {
+long long map_launch(SweepArgs& a, long long slots) {
     constexpr int T = sweep_threads(DIR);
     constexpr bool TMA = MFC_TMA_YZ && (FORM == FORM_MIXED || FORM == FORM_GATED) && (DIR == 1 || DIR == 2) && !NU;
-    SweepArgs a = a0;
-    const long long slots = sweep_slots<NDIM, DIR, MODE, FORM, NU, NF>();
     constexpr bool BAL = sweep_balanced(FORM, NF);
-    long long blocks;
     if (BAL && !(TMA && a.tmap)) {
         // balanced mapping: MFC_BAL_WAVES x the resident warps, each taking at
         // least MFC_BAL_MIN_CELLS cells
@@ -1145,19 +1144,44 @@ cudaError_t launch_kernel(const SweepArgs& a0, cudaStream_t s) {
         if (w > wmax) w = wmax;
         a.nwarps = w;
         a.seg = 0;
-        blocks = (w * 32 + T - 1) / T;
-    } else {
-        a.nwarps = 0;
-        a.seg = pick_seg(DIR, a.n, T, slots);
-        blocks = (sweep_warps(DIR, a.n, a.seg) * 32 + T - 1) / T;
+        return (w * 32 + T - 1) / T;
     }
+    a.nwarps = 0;
+    a.seg = pick_seg(DIR, a.n, T, slots);
+    return (sweep_warps(DIR, a.n, a.seg) * 32 + T - 1) / T;
+}
+
+template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF, bool LEAN>
+cudaError_t launch_mapped(const SweepArgs& a, long long blocks, cudaStream_t s) {
     if (blocks <= 0 || a.dry) return cudaSuccess;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     CUtensorMap tm;
     if (a.tmap) tm = *static_cast<const CUtensorMap*>(a.tmap);
     else memset(&tm, 0, sizeof(tm));
-    sweep_kernel<NDIM, DIR, MODE, FORM, NU, NF><<<(unsigned)blocks, T, 0, s>>>(a, tm);
+    sweep_kernel<NDIM, DIR, MODE, FORM, NU, NF, LEAN><<<(unsigned)blocks, sweep_threads(DIR), 0, s>>>(a, tm);
     return cudaGetLastError();
+}
+
+template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF>
+cudaError_t launch_kernel(const SweepArgs& a0, cudaStream_t s) {
+    constexpr LeanUse use = lean_use(FORM, NDIM, DIR, NU, NF);
+    SweepArgs a = a0;
+    LaunchFill lean{}, full{};
+    if constexpr (use != LEAN_NEVER) {
+        lean.slots = sweep_slots<NDIM, DIR, MODE, FORM, NU, NF, true>();
+        lean.blocks = map_launch<NDIM, DIR, MODE, FORM, NU, NF>(a, lean.slots);
+    }
+    SweepArgs b = a0;
+    if constexpr (use != LEAN_ALWAYS) {
+        full.slots = sweep_slots<NDIM, DIR, MODE, FORM, NU, NF, false>();
+        full.blocks = map_launch<NDIM, DIR, MODE, FORM, NU, NF>(b, full.slots);
+    }
+    if constexpr (use == LEAN_BY_LAUNCH) {
+        if (take_lean(NDIM, DIR, NU, NF, a0.order, lean, full))
+            return launch_mapped<NDIM, DIR, MODE, FORM, NU, NF, true>(a, lean.blocks, s);
+    }
+    if constexpr (use == LEAN_ALWAYS) return launch_mapped<NDIM, DIR, MODE, FORM, NU, NF, true>(a, lean.blocks, s);
+    else return launch_mapped<NDIM, DIR, MODE, FORM, NU, NF, false>(b, full.blocks, s);
 }
 
 // SSP-RK3 stage update from the finished accumulator (gated form, 3-D): D_k in
