@@ -293,8 +293,8 @@ def roofline_for(form, res, peak_alu, alu_src, hbm_peak, hbm_src):
     flops = flops_cell_dir(nf, 3, 3 if form.endswith("_weno3") else 5)
     if name == "sweep_y":
         flops += neq
-    if name == "sweep_z":
-        flops += flops_last_sweep_extra(nf, 3)
+    if name == "sweep_z":   # with the stage update, unless that is a kernel of its own
+        flops += neq if kt.get("stage_update", (0, 0))[1] else flops_last_sweep_extra(nf, 3)
     achieved = flops * ncell / avg_s / 1e12
     share = total_ms / sum(v[0] for v in kt.values())
     if base == "fp64":   # the reference-order form (no FMA contraction)

@@ -141,7 +141,10 @@ int mfc_set_timing(mfc_ctx* ctx, int enable);
 
 /* Kernel kind `index` (0-based): its name, the summed device time in ms and
  * the number of launches since timing was enabled.  Returns MFC_EINVAL when
- * index is out of range. */
+ * index is out of range.  Kinds: step_begin, sweep_x, sweep_y, sweep_z, and
+ * stage_update, which only the gated form in 3-D launches (elsewhere the last
+ * sweep applies the update); the launches of a step over all kinds add up to
+ * mfc_launches_per_step. */
 int mfc_kernel_time(mfc_ctx* ctx, int index, const char** name, double* ms, long long* launches);
 
 /* ---- gated form (MFC_GATED): the troubled-cell network ------------------

@@ -22,8 +22,8 @@ using namespace mfc5;
 
 namespace {
 
-enum KernelKind { K_STEP_BEGIN = 0, K_SWEEP_X, K_SWEEP_Y, K_SWEEP_Z, K_NKINDS };
-const char* kKindNames[K_NKINDS] = {"step_begin", "sweep_x", "sweep_y", "sweep_z"};
+enum KernelKind { K_STEP_BEGIN = 0, K_SWEEP_X, K_SWEEP_Y, K_SWEEP_Z, K_STAGE_UPDATE, K_NKINDS };
+const char* kKindNames[K_NKINDS] = {"step_begin", "sweep_x", "sweep_y", "sweep_z", "stage_update"};
 constexpr int kMaxTimedLaunches = 16;
 
 }  // namespace
@@ -366,28 +366,43 @@ static void stage_buffers(mfc_ctx* ctx, int k, SweepArgs& a) {
     a.qout2 = (k == 3 && fp32_state(ctx)) ? (void*)ctx->s0 : NULL;
 }
 
+// Launches one stage on stream s: a sweep per direction, the last of which
+// applies the stage update, or the update after it (split_update).  mark(kind)
+// follows each launch.
+template <typename Mark>
+static cudaError_t launch_stage(mfc_ctx* ctx, const SweepArgs& a, cudaStream_t s, Mark&& mark) {
+    const bool split = split_update(ctx->form, ctx->ndim);
+    cudaError_t e;
+    for (int d = 0; d < ctx->ndim; ++d) {
+        const int mode = d == ctx->ndim - 1 && !split ? SW_LAST_RK : (d == 0 ? SW_FIRST : SW_MID);
+        if ((e = launch_sweep(ctx, d, mode, a, s)) != cudaSuccess) return e;
+        if ((e = mark(K_SWEEP_X + d)) != cudaSuccess) return e;
+    }
+    if (!split) return cudaSuccess;
+    if ((e = launch_stage_update(ctx->ndim, a, s)) != cudaSuccess) return e;
+    return mark(K_STAGE_UPDATE);
+}
+
+// For mark where nothing follows a launch.
+static cudaError_t no_mark(int) { return cudaSuccess; }
+
 // Enqueue the launches of one step on stream s; with `timed`, bracket each
 // launch with events ev[i], ev[i+1] (recorded for later accumulation).
 static cudaError_t enqueue_step(mfc_ctx* ctx, cudaStream_t s, bool timed, int* kinds, int* nl) {
     int L = 0;
     cudaError_t e;
+    auto mark = [&](int kind) {
+        if (!timed) return cudaSuccess;
+        kinds[L++] = kind;
+        return cudaEventRecord(ctx->ev[L], s);
+    };
     if (timed && (e = cudaEventRecord(ctx->ev[0], s)) != cudaSuccess) return e;
     if ((e = launch_step_begin(ctx->ctrl, s)) != cudaSuccess) return e;
-    if (timed) {
-        kinds[L++] = K_STEP_BEGIN;
-        if ((e = cudaEventRecord(ctx->ev[L], s)) != cudaSuccess) return e;
-    }
+    if ((e = mark(K_STEP_BEGIN)) != cudaSuccess) return e;
     for (int k = 1; k <= 3; ++k) {
         SweepArgs a = base_args(ctx);
         stage_buffers(ctx, k, a);
-        for (int d = 0; d < ctx->ndim; ++d) {
-            int mode = d == ctx->ndim - 1 ? SW_LAST_RK : (d == 0 ? SW_FIRST : SW_MID);
-            if ((e = launch_sweep(ctx, d, mode, a, s)) != cudaSuccess) return e;
-            if (timed) {
-                kinds[L++] = K_SWEEP_X + d;
-                if ((e = cudaEventRecord(ctx->ev[L], s)) != cudaSuccess) return e;
-            }
-        }
+        if ((e = launch_stage(ctx, a, s, mark)) != cudaSuccess) return e;
     }
     if (nl) *nl = L;
     return cudaSuccess;
@@ -399,8 +414,7 @@ static int ensure_graph(mfc_ctx* ctx) {
     // rather than inside the capture
     SweepArgs dry = base_args(ctx);
     dry.dry = 1;
-    for (int d = 0; d < ctx->ndim; ++d)
-        CK(launch_sweep(ctx, d, d == ctx->ndim - 1 ? SW_LAST_RK : (d == 0 ? SW_FIRST : SW_MID), dry, ctx->stream));
+    CK(launch_stage(ctx, dry, ctx->stream, no_mark));
     cudaGraph_t g = NULL;
     CK(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = enqueue_step(ctx, ctx->cap_stream, false, NULL, NULL);
@@ -828,11 +842,7 @@ extern "C" int mfc_block_stage(mfc_ctx* ctx, int stage, const void* halo) {
     SweepArgs a = base_args(ctx);
     stage_buffers(ctx, stage, a);
     ctx->halo_cur = halo;
-    cudaError_t e = cudaSuccess;
-    for (int d = 0; d < ctx->ndim && e == cudaSuccess; ++d) {
-        int mode = d == ctx->ndim - 1 ? SW_LAST_RK : (d == 0 ? SW_FIRST : SW_MID);
-        e = launch_sweep(ctx, d, mode, a, ctx->stream);
-    }
+    const cudaError_t e = launch_stage(ctx, a, ctx->stream, no_mark);
     ctx->halo_cur = NULL;
     CK(e);
     return MFC_OK;

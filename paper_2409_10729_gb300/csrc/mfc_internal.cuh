@@ -151,6 +151,8 @@ constexpr int kGateParams = 1281;
 cudaError_t launch_sweep_mixed(int ndim, int dir, int mode, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_sweep_fp64x(int ndim, int dir, int mode, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_sweep_gated(int ndim, int dir, int mode, const SweepArgs& a, cudaStream_t s);
+// the stage update of a form and dimension whose sweeps do not apply it (split_update)
+cudaError_t launch_stage_update(int ndim, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_gate_samples(int ndim, const double* q, const int* n, const int* periodic, const Eos& e,
                                 double eps, float tau, float* X, float* Y, cudaStream_t s);
 

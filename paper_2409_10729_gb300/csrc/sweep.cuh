@@ -737,7 +737,7 @@ sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
         // reconstruct two fields at a time (packed FP32 pairs, physics.cuh), not in
         // 1-D, where one dependent chain per warp is all there is (2122 cells 4%
         // slower); from a table only along x, whose kernel has the registers
-        // (elsewhere they spill), and not in lean kernels
+        // (elsewhere they spill); lean kernels pack nothing on uniform grids
         constexpr bool TABP = DIR == 0 && NDIM > 1;
         constexpr bool PACK = !NU && NDIM > 1 && !LEAN;
         // mixed form, x sweep: the first differences d1..d3 and curvature parts C0, C1
@@ -1190,8 +1190,9 @@ cudaError_t launch_kernel(const SweepArgs& a0, cudaStream_t s) {
 // a kernel of its own it streams (172 to 256 bytes a cell at full occupancy),
 // and the z sweep runs as MID at the y sweep's three blocks per SM, where with the
 // update's operands beside stencil and network it had two.  Measured, sweep with
-// update -> sweep + update: gated 256^3 1.531 -> 1.211 ms, 96^3 0.170 -> 0.130,
-// 64^3 0.067 -> 0.071.  The mixed form, whose fused sweep has three blocks, does
+// update -> sweep + update: gated 256^3 1.531 -> 1.211 ms; whole steps 160^3 2.560 ->
+// 2.377 ms, 96^3 0.949 -> 0.866, 64^3 0.435 -> 0.416, 48^3 0.254 -> 0.256, 32^3 0.210
+// -> 0.208, 8^3 0.193 -> 0.189: no size needs the fused form.  The mixed form, whose fused sweep has three blocks, does
 // not gain (512^3 6.69 -> 6.81 ms, 160^3 0.274 -> 0.254, 96^3 0.057 -> 0.069): the
 // accumulator's extra 56 bytes a cell and the launch cost what it saves.
 template <int NDIM>
@@ -1249,15 +1250,6 @@ __global__ void __launch_bounds__(256) stage_update_kernel(const SweepArgs a) {
     }
 }
 
-template <int NDIM>
-cudaError_t launch_stage_update(const SweepArgs& a, cudaStream_t s) {
-    if (a.dry) return cudaSuccess;
-    long long blocks = (a.ncell + 255) / 256;
-    if (blocks > 152LL * 64) blocks = 152LL * 64;
-    stage_update_kernel<NDIM><<<(unsigned)blocks, 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
 // the FP64 form's sweep (tile.cuh)
 template <int NDIM, int DIR, int MODE, bool NU, int NF>
 cudaError_t launch_tile(const SweepArgs& a, cudaStream_t s);
@@ -1280,7 +1272,8 @@ cudaError_t launch_one(const SweepArgs& a, cudaStream_t s) {
 }
 
 // Launch one sweep: the valid (direction, mode) pairs are x FIRST, y MID
-// (3-D), and LAST_RK / LAST_RHS on the last direction.
+// (3-D), and LAST_RK / LAST_RHS on the last direction; where the stage update is a
+// kernel of its own (split_update), MID there instead of LAST_RK.
 template <int NDIM, int FORM, int NF>
 cudaError_t launch_sweep_t(int dir, int mode, const SweepArgs& a, cudaStream_t s) {
     constexpr int LAST = NDIM - 1;
@@ -1289,12 +1282,9 @@ cudaError_t launch_sweep_t(int dir, int mode, const SweepArgs& a, cudaStream_t s
     } else if (dir == 1 && mode == SW_MID && NDIM == 3) {
         if constexpr (NDIM == 3) return launch_one<NDIM, 1, SW_MID, FORM, NF>(a, s);
     } else if (dir == LAST && mode == SW_LAST_RK) {
-        if constexpr (split_update(FORM, NDIM)) {
-            const cudaError_t e = launch_one<NDIM, LAST, SW_MID, FORM, NF>(a, s);
-            return e != cudaSuccess ? e : launch_stage_update<NDIM>(a, s);
-        } else {
-            return launch_one<NDIM, LAST, SW_LAST_RK, FORM, NF>(a, s);
-        }
+        if constexpr (!split_update(FORM, NDIM)) return launch_one<NDIM, LAST, SW_LAST_RK, FORM, NF>(a, s);
+    } else if (dir == LAST && mode == SW_MID) {
+        if constexpr (split_update(FORM, NDIM)) return launch_one<NDIM, LAST, SW_MID, FORM, NF>(a, s);
     } else if (dir == LAST && mode == SW_LAST_RHS) {
         return launch_one<NDIM, LAST, SW_LAST_RHS, FORM, NF>(a, s);
     }

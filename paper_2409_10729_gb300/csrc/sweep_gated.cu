@@ -11,6 +11,16 @@ cudaError_t launch_sweep_gated(int ndim, int dir, int mode, const SweepArgs& a, 
     return launch_sweep_any<FORM_GATED>(ndim, dir, mode, a, s);
 }
 
+cudaError_t launch_stage_update(int ndim, const SweepArgs& a, cudaStream_t s) {
+    static_assert(split_update(FORM_GATED, 3), "the one split update");
+    if (ndim != 3) return cudaErrorInvalidValue;
+    if (a.dry) return cudaSuccess;
+    long long blocks = (a.ncell + 255) / 256;
+    if (blocks > 152LL * 64) blocks = 152LL * 64;
+    stage_update_kernel<3><<<(unsigned)blocks, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 // Batched logits with the sweep's tensor-core evaluation: each warp takes 64
 // samples per pass (rows 0-31 in the density slot, 32-63 in the pressure slot).
 __global__ void __launch_bounds__(128) gate_forward_tc_kernel(const float* __restrict__ X, long long n,
