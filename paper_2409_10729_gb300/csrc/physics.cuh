@@ -84,16 +84,11 @@ __device__ __forceinline__ bool pos(R x) {
     if constexpr (sizeof(R) == 8) return gt0(x);
     else return x > R(0);
 }
+
 template <typename R>
-__device__ __forceinline__ bool nonneg(R x) {
-    if constexpr (sizeof(R) == 8) return ge0(x);
-    else return R(0) <= x;
-}
+__device__ __forceinline__ bool nonneg(R x) { return R(0) <= x; }
 template <typename R>
-__device__ __forceinline__ bool lt(R a, R b) {
-    if constexpr (sizeof(R) == 8) return less(a, b);
-    else return a < b;
-}
+__device__ __forceinline__ bool lt(R a, R b) { return a < b; }
 
 // Mixture density of the partial densities w[0..NF-1].
 template <int NF, typename R>
@@ -110,28 +105,18 @@ __device__ __forceinline__ R rdiv(R a, R b) { return a / b; }
 template <typename R>
 __device__ __forceinline__ R sqrt_pos(R x) { return sqrt(x); }
 
-// EOS constants in the working precision R (converted once per thread, so the
-// FP32 path issues no FP64 conversions per face).
+// EOS constants of the FP32 forms in registers.
 template <typename R, int NF = 2>
 struct EosR {
+    static_assert(sizeof(R) == 4, "the FP64 form reads Eos itself");
     R dg[NF - 1], gN, dP[NF - 1], PN;
     __device__ __forceinline__ explicit EosR(const Eos& e) {
-        if constexpr (sizeof(R) == 4) {
-            gN = e.g32[NF - 1];
-            PN = e.P32[NF - 1];
-        } else {
-            gN = R(e.g[NF - 1]);
-            PN = R(e.P[NF - 1]);
-        }
+        gN = e.g32[NF - 1];
+        PN = e.P32[NF - 1];
 #pragma unroll
         for (int i = 0; i < NF - 1; ++i) {
-            if constexpr (sizeof(R) == 4) {
-                dg[i] = e.dg32[i];
-                dP[i] = e.dP32[i];
-            } else {
-                dg[i] = R(e.dg[i]);
-                dP[i] = R(e.dP[i]);
-            }
+            dg[i] = e.dg32[i];
+            dP[i] = e.dP32[i];
         }
     }
 };

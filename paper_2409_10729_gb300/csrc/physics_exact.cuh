@@ -534,7 +534,7 @@ __device__ __forceinline__ void weno5_tc(double eps, double v0, double v1, doubl
     r1 = p[2];
 }
 
-// The right-face candidates r0, r1 of the cell whose window is v0..v3 (as in weno5_t).
+// The right-face candidates r0, r1 of the cell whose window is v0..v3 (as in weno5_tc).
 __device__ __forceinline__ void weno5_right01(double v0, double v1, double v2, double v3, double& r0, double& r1) {
     r0 = div6(fma2(2.0, v2, -v0 + mul_small<5>(v1)));
     r1 = div6(fma2(2.0, v1, mul_small<5>(v2)) - v3);

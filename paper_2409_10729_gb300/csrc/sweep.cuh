@@ -29,8 +29,6 @@
 
 #include <string.h>
 
-#include <type_traits>
-
 #include "mfc.h"
 #include "mfc_internal.cuh"
 #include "physics_exact.cuh"
@@ -46,15 +44,13 @@ __device__ __forceinline__ int bc_index(int j, int n, int periodic) {
     return j < 0 ? 0 : n - 1;
 }
 
-// Fields a sweep reads per cell, in load order.  FP64: the conservative
-// state.  Mixed: the FP32 state with the pressure stored as field NEQ (formed
-// in FP64 when the state was written) read in place of rho E.
-template <int NDIM, typename R, int NF = 2>
+// Fields a sweep reads per cell, in load order: the FP32 state with the pressure
+// stored as field NEQ (formed in FP64 when the state was written) read in place
+// of rho E.
+template <int NDIM, int NF = 2>
 struct LoadSet {
     static constexpr int N = Fields<NDIM, NF>::NEQ;
-    __device__ static constexpr int field(int k) {
-        return (sizeof(R) == 8 || k != Fields<NDIM, NF>::IE) ? k : N;
-    }
+    __device__ static constexpr int field(int k) { return k != Fields<NDIM, NF>::IE ? k : N; }
 };
 
 // Primitives from the loaded values v[] (see LoadSet).
@@ -142,7 +138,7 @@ __device__ __forceinline__ R cell_wavespeed(const EosR<R, NF>& e, const R* w, co
     R s = R(0);
 #pragma unroll
     for (int d = 0; d < NDIM; ++d) s += (fabs(w[FL::IU + d]) + c) * R(inv_dx[d]);
-    bad |= !lt(s, R(INFINITY));
+    bad |= !(s < R(INFINITY));
     return s;
 }
 
@@ -177,9 +173,6 @@ struct XStage {
     static constexpr int CH = 32 / sizeof(R);   // cells per row and sector along x
     static constexpr int PITCH = CH + 1;        // padded row pitch (conflict-free accesses)
 };
-
-template <int FORM>
-using FormReal = typename std::conditional<FORM == FORM_MIXED || FORM == FORM_GATED, float, double>::type;
 
 // ---- gate network on the tensor cores, FP32-accurate ----------------------
 // A warp evaluates the network for its 32 cells x 2 sensors = 64 samples at
@@ -510,10 +503,10 @@ constexpr int sweep_min_blocks() {
 template <int NDIM, int DIR, int MODE, int FORM, bool NU, int NF, bool LEAN>
 __global__ void __launch_bounds__(sweep_threads(DIR), sweep_min_blocks<FORM, MODE, DIR, NF, NDIM, NU, LEAN>())
 sweep_kernel(const SweepArgs a, const __grid_constant__ CUtensorMap tmap) {
-    using R = FormReal<FORM>;
+    using R = float;
     constexpr bool GATED = FORM == FORM_GATED;
     using FL = Fields<NDIM, NF>;
-    using LS = LoadSet<NDIM, R, NF>;
+    using LS = LoadSet<NDIM, NF>;
     constexpr int NEQ = FL::NEQ, IE = FL::IE, IA = FL::IA, NA = FL::NA;
     constexpr int NL = LS::N;
     constexpr int CH = XStage<R>::CH, PITCH = XStage<R>::PITCH;
