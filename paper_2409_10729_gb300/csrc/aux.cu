@@ -31,7 +31,8 @@ static unsigned aux_blocks(long long n) {
 // products are integer ones too (exact::MulInt).  Measured, 512^3 mixed, the
 // call: 27.8 ms as four kernels with FP64 divisions, 14.1 fused with integer
 // quotients and roots (FP64 pipe 84% busy), 12.8 with integer products at three
-// blocks per SM (128 registers, two blocks: 18.6).
+// blocks per SM (128 registers, two blocks: 18.6); 13.7 now that quotients and
+// products take any normal operand (physics_exact.cuh, quot).
 template <int NDIM, int NF, bool PRIM, bool MIXED>
 __global__ void __launch_bounds__(kAuxThreads, 3)
 set_state_kernel(const double* src, double* qn, float* __restrict__ s0, long long nc, Eos e, double dx0, double dx1,

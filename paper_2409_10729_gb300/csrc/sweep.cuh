@@ -8,7 +8,8 @@
 //   L_d = (F_{i-1/2} - F_{i+1/2}) / dx_d  (+ alpha1_i (u_f,i+1/2 - u_f,i-1/2) / dx_d)
 // which it stores into, adds to, or finishes the RHS accumulator with.  The
 // last direction's sweep also applies the SSP-RK3 stage update and, on the
-// third stage, reduces the CFL wave speed of the new state.
+// third stage, reduces the CFL wave speed of the new state (gated form in 3-D:
+// stage_update_kernel does).
 //
 // Thread mapping.  A warp owns 32 adjacent pencils along d and a segment of
 // `seg` cells of each -- or, in the balanced split, an even share of all the

@@ -18,12 +18,14 @@
 // field at a time from shared memory needs 100, 16 warps, and reaches 80 to 84%
 // (128^3, ncu: 547 FP64 of 9975 instructions per 32 cells and 0.96 issued per
 // clock with WENO's and HLLC's quotients on the integer pipes; 440 and 1.7 with
-// WENO's products and HLLC's square roots there too).  It also gives small grids parallel work: a thread's serial chain is
-// R reconstructions and one flux instead of a segment of whole cells, and a
-// single pencil fills its warps with cells along it.  Measured, sliding window
+// WENO's products and HLLC's square roots there too).  It also gives small grids
+// parallel work: a thread's serial chain is R reconstructions and one flux
+// instead of a segment of whole cells, and a single pencil fills its warps with
+// cells along it.  Measured, sliding window
 // -> tiles: 256^3 droplets 0.557 -> 0.464 ns per cell, equation and RHS;
 // 1024x512 column 6.72 -> 3.36 ms a step; 32^3 RHS 3.9 -> 0.18 ms; 1000-cell
-// tube 2.67 -> 0.041 ms a step.  (256^3 0.411 now, physics_exact.cuh.)
+// tube 2.67 -> 0.041 ms a step.  (256^3 0.39 now, with WENO's products off the
+// FP64 pipe too, physics_exact.cuh, and the shapes of pick_tile.)
 #pragma once
 #include <algorithm>
 #include <atomic>
