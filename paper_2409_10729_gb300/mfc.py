@@ -365,9 +365,10 @@ class Solver:
 
 def _stream() -> int:
     import torch
-    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # not a public name
-    device = torch.cuda.current_device()
-    return raw(device) if raw else torch.cuda.current_stream(device).cuda_stream
+    try:   # not a public name
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    except AttributeError:
+        return torch.cuda.current_stream(torch.cuda.current_device()).cuda_stream
 
 
 def mlp_loss_grad(X, Y, theta, grad, loss, pos_weight: float = 1.0):
