@@ -245,7 +245,9 @@ __host__ __device__ constexpr bool sweep_balanced(int form, int nf) {
 #define MFC_MIN_BLOCKS_GATED 3
 #endif
 // the gated y sweep fits 168 registers since its pairs are packed (256^3 0.917 ->
-// 0.794 ms); x and the stage update do not gain (x 0.929 -> 1.073)
+// 0.794 ms); x and the stage update do not gain (x 0.929 -> 1.073), nor does the last
+// sweep of a 2-D right-hand side (us a call at two blocks -> three: 200x150 71.8 ->
+// 78.4, 256x128 74.3 -> 78.4, 320x160 76.7 -> 78.4, 640x320 127, 2048x1024 646 -> 658)
 #ifndef MFC_MIN_BLOCKS_GATED_X
 #define MFC_MIN_BLOCKS_GATED_X 2
 #endif

@@ -492,7 +492,7 @@ constexpr int sweep_min_blocks() {
     constexpr int per128 = FORM == FORM_MIXED   ? (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_MIXED_RK
                                                    : DIR == 0         ? ((NU || NDIM == 2) && !LEAN ? MFC_MIN_BLOCKS_MIXED_X3 : MFC_MIN_BLOCKS_MIXED_X)
                                                                       : MFC_MIN_BLOCKS_MIXED)
-                                                : (MODE == SW_LAST_RK ? MFC_MIN_BLOCKS_GATED_RK
+                                                : (MODE == SW_LAST_RK || (MODE == SW_LAST_RHS && NDIM == 2) ? MFC_MIN_BLOCKS_GATED_RK
                                                    : DIR == 0       ? MFC_MIN_BLOCKS_GATED_X
                                                                     : MFC_MIN_BLOCKS_GATED);
     return per128 * 128 / sweep_threads(DIR);
