@@ -142,7 +142,8 @@ constexpr int kTmaCells = 4;
 enum Form { FORM_MIXED = 1, FORM_FP64_EXACT = 2, FORM_GATED = 3 };
 
 // The stage update runs as a kernel of its own after the last sweep (sweep.cuh,
-// stage_update_kernel) instead of inside it.
+// stage_update_kernel) instead of inside it: gated form in 3-D, at every size (the
+// measurements are there).
 __host__ __device__ constexpr bool split_update(int form, int ndim) { return form == FORM_GATED && ndim == 3; }
 
 // Number of parameters of the gate network (W1[32][5], b1, W2[32][32], b2, w3, b3).
@@ -182,7 +183,7 @@ cudaError_t launch_pack_side(const void* q, void* out, int elem, int nfields, lo
 cudaError_t launch_block_begin(DevCtrl* ctrl, double dt, cudaStream_t s);
 cudaError_t run_fma_probe(int fp64, double* tflops, cudaStream_t s);
 
-// thread-block size of every sweep launch
+// thread-block size of the FP32 y and z sweeps (the FP64 tiles: kTileThreads)
 constexpr int kSweepThreads = 128;
 // threads per block of the sweep along direction d
 __host__ __device__ constexpr int sweep_threads(int dir) { return dir == 0 ? 32 : kSweepThreads; }
@@ -296,14 +297,14 @@ inline bool take_lean(int ndim, int dir, bool nu, int nf, int order, const Launc
     return 2 * full.blocks <= full.slots;
 }
 
-// 1: the sweeps issue the loads of the cell entering the stencil window at the
-// top of each step along the pencil (they complete under that step's
-// arithmetic); 0: at the bottom, just before they are used.
 // mixed form, uniform grids, x sweep: carry WENO5 first differences and
 // curvature parts from cell to cell (1) or form them in every cell (0)
 #ifndef MFC_DIFF_CARRY
 #define MFC_DIFF_CARRY 1
 #endif
+// 1: the FP32 sweeps issue the loads of the cell entering the stencil window at
+// the top of each step along the pencil (they complete under that step's
+// arithmetic); 0: at the bottom, just before they are used.
 #ifndef MFC_PREFETCH
 #define MFC_PREFETCH 1
 #endif

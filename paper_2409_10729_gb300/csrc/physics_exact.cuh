@@ -159,8 +159,9 @@ __device__ __forceinline__ bool normal_hi(unsigned h) { return (h & 0x7ff00000u)
 
 // RN(x^2) for |x| within 2^-300 .. 2^300; smaller x give 0, larger ones and NaN
 // clear ok.  (The squares of differences below 2^-300 are parts of smoothness
-// indicators, added to an eps whose own square is a normal number, at least
-// 2^-511: they are below half a unit in the last place of any such sum.)
+// indicators, added to eps.  They sum to less than 2^-598, under half a unit in
+// the last place of any eps from 2^-538 up; the square of a smaller eps is zero,
+// and the face values of such a cell are NaN with or without these parts.)
 __device__ __forceinline__ double sq_i(double x, bool& ok) {
     const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu, l = (unsigned)__double2loint(x);
     ok = ok && h < (1323u << 20);
