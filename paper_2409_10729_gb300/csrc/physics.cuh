@@ -200,12 +200,14 @@ __device__ __forceinline__ void weno5_dc(float v2, float d1, float d2, float d3,
 // multiply and fused multiply-add round each half as the scalar operation does.
 // They take two slots of the FMA pipe but one issue slot, and instruction issue
 // and latency bound the FP32 sweeps, not the FMA pipe (0.3 busy): 160^3, warp
-// instructions per 32 cells x 770 -> 648, y 846 -> 703, z 1283 -> 1150 with WENO
+// instructions per 32 cells x 770 -> 658, y 846 -> 703, z 1283 -> 1128 with WENO
 // packed.  Measured, mixed 512^3: x 3.77 -> 3.41 ms, y 3.24 -> 3.02, z 6.91 -> 6.69;
 // gated 256^3, with the linear reconstruction packed as well and the normalised
 // stencils formed only where the network runs, 10.38 -> 9.71 ms a step.  Each
 // function writes out, operation for operation, what the compiler makes of the
-// scalar one (which a*b + c*d product is fused), so the results keep their bits.
+// scalar one (which a*b + c*d product is fused), so the results keep their bits
+// (gated form in 3-D: all but 2 of the 117 million right-hand-side values of 256^3
+// droplets after one step, a last place of a momentum residue of 1e-10).
 // The tabulated reconstruction of non-uniform grids forms its table sums field by
 // field -- one load of a table value serves all fields -- and packs what follows
 // in the x sweep only (192^3 0.370 -> 0.344 ms, 0.309 at three blocks per SM); y and
